@@ -31,6 +31,10 @@ size_t rollout_smem_bytes(int B, int V, int R, bool head, int grid) {
          static_cast<size_t>(B) * rollout_rows_per_cta(V, R, head, grid) * sizeof(float);
 }
 
+// Shared memory of h_j of every sequence (two-barrier steps): whole 256-unit runs (h_slot), and 16
+// bytes for its alignment.
+static long long h_bytes(const RolloutParams& p) { return static_cast<long long>(p.B) * ((p.Ds + 255) / 256 * 256) * 4 + 16; }
+
 // Two grid barriers per step (phase A done by every CTA for all units, gates_all / ub_phase):
 // the resident kernel with a table, when h_j of every sequence fits in shared memory beside u and
 // the base logits (the shared-memory W2 rows give way to it).
@@ -38,34 +42,36 @@ static bool use_fast_gates(const RolloutParams& p, int grid) {
   // gates_all reads the biases four at a time (8-byte loads)
   const bool bias_ok = (reinterpret_cast<uintptr_t>(p.b_ih) & 7u) == 0 && (reinterpret_cast<uintptr_t>(p.b_hh) & 7u) == 0;
   return use_resident(p) && p.x_table && p.uh && p.gh && p.ucount && p.uhcount && p.Ds <= 1024 && bias_ok &&
-         resident_smem_rows(p.B, p.V, p.R, grid, static_cast<long long>(p.B) * p.Ds * 4 + 16) >= 0;
+         resident_smem_rows(p.B, p.V, p.R, grid, h_bytes(p)) >= 0;
 }
 
-// Phase C on the tensor cores (two-barrier steps, at most two sequences, r a multiple of 64 up to
-// 256): the 128-row blocks of a CTA's rows, tb in tensor memory and sb in shared memory, that
-// cover the most rows (tensor memory first: an A block there costs r/2 columns and its D 16 more;
-// one in shared memory costs 128 r bf16 beside the fixed buffers).  False when the layout does
-// not apply or would leave more than kMmaMaxL2Rows rows of a CTA to read through L2 every step.
+// Phase C on the tensor cores (r a multiple of 64 up to 256): the 128-row blocks of a CTA's rows,
+// tb in tensor memory and sb in shared memory, that cover the most rows (tensor memory first: an A
+// block there costs r/2 columns and its D mma_n(B) more; one in shared memory costs 128 r bf16
+// beside the fixed buffers).  False when the layout does not apply: the inverse-CDF rule beyond the
+// table's two sequences (its draw is decided by the order of the fp32 sums, which the CUDA-core
+// layout keeps), or that rule with more than kMmaMaxL2Rows rows of a CTA left to read through L2.
 static bool mma_blocks(const RolloutParams& p, int grid, int* tb, int* sb, size_t* smem) {
   *tb = *sb = 0;
-  if (!use_fast_gates(p, grid) || p.B > 2 || p.R % 64 != 0 || p.R > 256) return false;
+  if (!use_resident(p) || p.R % 64 != 0 || p.R > 256) return false;
+  if (p.uniforms && !(p.fast_gates && p.B <= 2)) return false;
   const int rows_cta = resident_rows_per_cta(p.V, grid);
-  const int need = (rows_cta + 127) / 128;
-  const long long fixed = 1024 + static_cast<long long>(p.R / 64) * kMmaBopTileBytes +
+  const int need = (rows_cta + 127) / 128, n = mma_n(p.B);
+  const long long fixed = 1024 + static_cast<long long>(p.R / 64) * n * 128 +
                           static_cast<long long>(p.B) * p.R * 4 + static_cast<long long>(p.B + 1) * rows_cta * 4 +
-                          static_cast<long long>(p.B) * p.Ds * 4 + 16;
+                          (p.fast_gates ? h_bytes(p) : 0);
   const long long blk = static_cast<long long>(p.R / 64) * kMmaTileBytes;
   if (fixed > static_cast<long long>(kRollMaxSmem)) return false;
   const int s_max = static_cast<int>((static_cast<long long>(kRollMaxSmem) - fixed) / blk);
   int bt = 0, bs = 0;
   for (int t = 0; t <= need; ++t) {
     const int room = kTmemCols - t * (p.R / 2);  // columns left for the D blocks
-    if (room < 16 * t) break;
-    const int s = std::min(std::min(s_max, need - t), room / 16 - t);
+    if (room < n * t) break;
+    const int s = std::min(std::min(s_max, need - t), room / n - t);
     if (s < 0) continue;
     if (t + s > bt + bs || (t + s == bt + bs && t > bt)) { bt = t; bs = s; }
   }
-  if (bt + bs == 0 || rows_cta - 128 * (bt + bs) > kMmaMaxL2Rows) return false;
+  if (bt + bs == 0 || (p.uniforms && rows_cta - 128 * (bt + bs) > kMmaMaxL2Rows)) return false;
   *tb = bt;
   *sb = bs;
   *smem = static_cast<size_t>(fixed + bs * blk);
@@ -83,20 +89,20 @@ cudaError_t launch_rollout(const RolloutParams& p, int grid, cudaStream_t stream
   pp.fast_gates = use_fast_gates(p, grid) ? 1 : 0;
   pp.mma_tb = pp.mma_sb = 0;
   if (pp.fast_gates) {
-    const long long hbytes = static_cast<long long>(p.B) * p.Ds * 4 + 16;  // + alignment of s_h
+    const long long hbytes = h_bytes(p);
     pp.smem_rows = resident_smem_rows(p.B, p.V, p.R, grid, hbytes);
     smem = static_cast<size_t>(pp.smem_rows) * p.R * 2 + static_cast<size_t>(p.B) * p.R * 4 +
            static_cast<size_t>(p.B + 1) * resident_rows_per_cta(p.V, grid) * 4 + static_cast<size_t>(hbytes);
-    int tb = 0, sb = 0;
-    size_t mma_smem = 0;
-    if (tm_w2 != nullptr && mma_blocks(pp, grid, &tb, &sb, &mma_smem)) {
-      pp.mma_tb = tb;
-      pp.mma_sb = sb;
-      pp.smem_rows = 0;
-      smem = mma_smem;
-    }
-    if (smem > kRollMaxSmem) return cudaErrorInvalidValue;
   }
+  int tb = 0, sb = 0;
+  size_t mma_smem = 0;
+  if (tm_w2 != nullptr && mma_blocks(pp, grid, &tb, &sb, &mma_smem)) {
+    pp.mma_tb = tb;
+    pp.mma_sb = sb;
+    pp.smem_rows = 0;
+    smem = mma_smem;
+  }
+  if (smem > kRollMaxSmem) return cudaErrorInvalidValue;
   if (!use_resident(p)) pp.uh = nullptr;  // only the resident kernel computes it before its steps
   CUtensorMap tm;
   if (tm_w2 != nullptr) tm = *tm_w2;

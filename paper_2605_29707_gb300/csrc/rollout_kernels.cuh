@@ -65,6 +65,15 @@ __device__ __forceinline__ void tc_mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem,
       : "memory");
 }
 
+// D (16x8, f32) += A (16x16 bf16, row-major) * B (16x8 bf16, column-major)
+__device__ __forceinline__ void mma_sync_16816(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
 // Makes this thread's ordinary shared-memory writes visible to the tensor core (async proxy);
 // a thread barrier must follow before the MMA that reads them is issued.
 __device__ __forceinline__ void fence_proxy_async_smem() {
@@ -79,6 +88,16 @@ __device__ __forceinline__ void tc_ld_x4(uint32_t taddr, float (&v)[4]) {
                : "r"(taddr));
 #pragma unroll
   for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Each thread of the warp reads 8 consecutive 32-bit columns of its TMEM lane.
+__device__ __forceinline__ void tc_ld_x8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ float bf2f(__nv_bfloat16 x) { return __bfloat162float(x); }
@@ -137,6 +156,9 @@ __device__ __forceinline__ void tc_st_x16(uint32_t taddr, const uint32_t (&r)[16
 
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
 // 4-byte asynchronous copy global -> shared (completes at cp_async_wait_all)
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
@@ -235,6 +257,15 @@ __device__ __forceinline__ void lse_push(Lse& a, float x, int id) {
   } else {
     a.s += __expf(x - a.m);
   }
+}
+
+// a's sum of exp relative to m >= a.m (0 when a is empty).
+__device__ __forceinline__ float lse_scaled(const Lse& a, float m) {
+  return a.m == -INFINITY ? 0.f : a.m == m ? a.s : a.s * __expf(a.m - m);
+}
+
+__device__ __forceinline__ float f32_unord(uint32_t o) {  // the inverse of f32_ord
+  return __uint_as_float((o & 0x80000000u) ? (o & 0x7FFFFFFFu) : ~o);
 }
 
 __device__ __forceinline__ void lse_merge(Lse& a, const Lse& b) {
@@ -468,45 +499,70 @@ __device__ __forceinline__ void bf4(const __nv_bfloat16* p, float (&f)[4]) {
   f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y;
 }
 
+// Where unit c of a sequence's h_j lies in the CTA's shared memory: within each run of 256 units the
+// lower halves (4 units) of the lanes' 8-unit groups come first, then the upper halves, so that a
+// warp's two 16-byte reads of its groups (ub_rows) touch every bank once each.
+__device__ __forceinline__ int h_slot(int c) { return (c & ~255) | ((c & 4) << 5) | ((c & 0xF8) >> 1) | (c & 3); }
+
 // ---- phase A with the input-projection table, two barriers per step (resident kernel): every
 //      CTA computes h_j of every unit and sequence itself, so that no grid barrier follows.  The
 //      input-gate sums are row t_j of the table, the recurrent sums W_hh h_{j-1} were computed in
 //      the previous step's phase B (gh; none at j = 0), and h_{j-1} is the CTA's own copy in
 //      shared memory, updated in place (unit q of h_j needs unit q of h_{j-1} only); four consecutive
-//      units per thread, every load of them issued before any arithmetic.
-__device__ __forceinline__ void gates_all(const RolloutParams& p, int j, const int* s_tok, float* s_h) {
+//      units per thread and sequence.  Bound by the latency of those loads through L2, so a thread
+//      issues the loads of up to four sequences before any arithmetic (one round trip instead of
+//      one a sequence: 5.3 -> 2.7 us a step at B = 4, H = 4096).
+template <int KB>
+__device__ __forceinline__ void gates_all(const RolloutParams& p, int j, const int* s_tok, float* s_h, int hs) {
+  constexpr int kU = KB < 4 ? KB : 4;  // (sequence, unit quad) items whose loads are in flight together
   const int B = p.B, Ds = p.Ds, D4 = Ds / 4;
   const float* gh = p.gh + static_cast<size_t>((j + 1) & 1) * B * 3 * Ds;  // W_hh h_{j-1}
-  for (int e = threadIdx.x; e < B * D4; e += kRollThreads) {
-    const int b = e / D4, q = (e - b * D4) * 4;
-    const float* xt = p.x_table + static_cast<size_t>(s_tok[b]) * 3 * Ds;
-    float4 x[3], hh[3];
-    float bi[3][4], bh[3][4];
+  for (int e0 = threadIdx.x; e0 < B * D4; e0 += kU * kRollThreads) {
+    float4 x[kU][3], hh[kU][3];
 #pragma unroll
-    for (int g = 0; g < 3; ++g) {
-      x[g] = __ldg(reinterpret_cast<const float4*>(xt + g * Ds + q));
-      // written by other CTAs in this launch: read through L2
-      hh[g] = j > 0 ? __ldcg(reinterpret_cast<const float4*>(gh + static_cast<size_t>(b) * 3 * Ds + g * Ds + q))
-                    : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (p.b_ih) bf4(p.b_ih + g * Ds + q, bi[g]); else bi[g][0] = bi[g][1] = bi[g][2] = bi[g][3] = 0.f;
-      if (p.b_hh) bf4(p.b_hh + g * Ds + q, bh[g]); else bh[g][0] = bh[g][1] = bh[g][2] = bh[g][3] = 0.f;
-    }
-    float* hrow = s_h + static_cast<size_t>(b) * Ds + q;
-    const float4 hp = j > 0 ? *reinterpret_cast<const float4*>(hrow) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float xa[3][4] = {{x[0].x, x[0].y, x[0].z, x[0].w}, {x[1].x, x[1].y, x[1].z, x[1].w},
-                            {x[2].x, x[2].y, x[2].z, x[2].w}};
-    const float ha[3][4] = {{hh[0].x, hh[0].y, hh[0].z, hh[0].w}, {hh[1].x, hh[1].y, hh[1].z, hh[1].w},
-                            {hh[2].x, hh[2].y, hh[2].z, hh[2].w}};
-    const float hpa[4] = {hp.x, hp.y, hp.z, hp.w};
-    float out[4];
+    for (int i = 0; i < kU; ++i) {
+      const int e = e0 + i * kRollThreads;
+      if (e < B * D4) {
+        const int b = e / D4, q = (e - b * D4) * 4;
+        const float* xt = p.x_table + static_cast<size_t>(s_tok[b]) * 3 * Ds;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float r = 1.f / (1.f + expf(-(xa[0][i] + bi[0][i] + ha[0][i] + bh[0][i])));
-      const float z = 1.f / (1.f + expf(-(xa[1][i] + bi[1][i] + ha[1][i] + bh[1][i])));
-      const float n = tanhf(xa[2][i] + bi[2][i] + r * (ha[2][i] + bh[2][i]));
-      out[i] = (1.f - z) * n + z * hpa[i];
+        for (int g = 0; g < 3; ++g) {
+          x[i][g] = __ldg(reinterpret_cast<const float4*>(xt + g * Ds + q));
+          // written by other CTAs in this launch: read through L2
+          hh[i][g] = j > 0 ? __ldcg(reinterpret_cast<const float4*>(gh + static_cast<size_t>(b) * 3 * Ds + g * Ds + q))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
     }
-    *reinterpret_cast<float4*>(hrow) = make_float4(out[0], out[1], out[2], out[3]);
+#pragma unroll
+    for (int i = 0; i < kU; ++i) {
+      const int e = e0 + i * kRollThreads;
+      if (e < B * D4) {
+        const int b = e / D4, q = (e - b * D4) * 4;
+        float bi[3][4], bh[3][4];
+#pragma unroll
+        for (int g = 0; g < 3; ++g) {
+          if (p.b_ih) bf4(p.b_ih + g * Ds + q, bi[g]); else bi[g][0] = bi[g][1] = bi[g][2] = bi[g][3] = 0.f;
+          if (p.b_hh) bf4(p.b_hh + g * Ds + q, bh[g]); else bh[g][0] = bh[g][1] = bh[g][2] = bh[g][3] = 0.f;
+        }
+        float* hrow = s_h + static_cast<size_t>(b) * hs + h_slot(q);
+        const float4 hp = j > 0 ? *reinterpret_cast<const float4*>(hrow) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float xa[3][4] = {{x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w}, {x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w},
+                                {x[i][2].x, x[i][2].y, x[i][2].z, x[i][2].w}};
+        const float ha[3][4] = {{hh[i][0].x, hh[i][0].y, hh[i][0].z, hh[i][0].w}, {hh[i][1].x, hh[i][1].y, hh[i][1].z, hh[i][1].w},
+                                {hh[i][2].x, hh[i][2].y, hh[i][2].z, hh[i][2].w}};
+        const float hpa[4] = {hp.x, hp.y, hp.z, hp.w};
+        float out[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const float r = 1.f / (1.f + expf(-(xa[0][v] + bi[0][v] + ha[0][v] + bh[0][v])));
+          const float z = 1.f / (1.f + expf(-(xa[1][v] + bi[1][v] + ha[1][v] + bh[1][v])));
+          const float n = tanhf(xa[2][v] + bi[2][v] + r * (ha[2][v] + bh[2][v]));
+          out[v] = (1.f - z) * n + z * hpa[v];
+        }
+        *reinterpret_cast<float4*>(hrow) = make_float4(out[0], out[1], out[2], out[3]);
+      }
+    }
   }
 }
 
@@ -521,7 +577,7 @@ __device__ __forceinline__ void gates_all(const RolloutParams& p, int j, const i
 //      issued before the arithmetic (Ds <= 1024: at most 4 chunks of 8 columns per lane and row).
 // count_u: each finished row of u is counted in p.ucount here (otherwise the caller counts them).
 template <int KB, int NR>
-__device__ __forceinline__ void ub_rows(const RolloutParams& p, int j, const float* s_h, int row0, int stride,
+__device__ __forceinline__ void ub_rows(const RolloutParams& p, int j, const float* s_h, int hs, int row0, int stride,
                                         int rows, int lane, uint64_t pol, bool count_u = true) {
   const int B = p.B, K = p.K, H = p.H, Ds = p.Ds, R = p.R;
   float* gh = p.gh + static_cast<size_t>(j & 1) * B * 3 * Ds;
@@ -565,11 +621,11 @@ __device__ __forceinline__ void ub_rows(const RolloutParams& p, int j, const flo
       wraw[k][i] = (w != nullptr && c < Ds) ? ld16_hint(w + c, pol) : make_uint4(0, 0, 0, 0);
     }
   }
-  float acc[NR][KB];
+  // the sums of (row k, sequence b) in entry k KB + b (three rows: a fourth of zeros)
+  constexpr int kV = (NR == 3 ? 4 : NR) * KB;
+  float acc[kV];
 #pragma unroll
-  for (int k = 0; k < NR; ++k)
-#pragma unroll
-    for (int b = 0; b < KB; ++b) acc[k][b] = 0.f;
+  for (int v = 0; v < kV; ++v) acc[v] = 0.f;
 #pragma unroll
   for (int i = 0; i < kCh; ++i) {
     const int c = lane * 8 + 256 * i;
@@ -580,40 +636,45 @@ __device__ __forceinline__ void ub_rows(const RolloutParams& p, int j, const flo
 #pragma unroll
     for (int b = 0; b < KB; ++b) {
       if (b < B) {
-        const float4 h0 = *reinterpret_cast<const float4*>(s_h + static_cast<size_t>(b) * Ds + c);
-        const float4 h1 = *reinterpret_cast<const float4*>(s_h + static_cast<size_t>(b) * Ds + c + 4);
+        const float* hb = s_h + static_cast<size_t>(b) * hs + 256 * i + lane * 4;  // h_slot(c), h_slot(c + 4)
+        const float4 h0 = *reinterpret_cast<const float4*>(hb);
+        const float4 h1 = *reinterpret_cast<const float4*>(hb + 128);
 #pragma unroll
         for (int k = 0; k < NR; ++k)
-          acc[k][b] += wv[k][0] * h0.x + wv[k][1] * h0.y + wv[k][2] * h0.z + wv[k][3] * h0.w +
-                       wv[k][4] * h1.x + wv[k][5] * h1.y + wv[k][6] * h1.z + wv[k][7] * h1.w;
+          acc[k * KB + b] += wv[k][0] * h0.x + wv[k][1] * h0.y + wv[k][2] * h0.z + wv[k][3] * h0.w +
+                             wv[k][4] * h1.x + wv[k][5] * h1.y + wv[k][6] * h1.z + wv[k][7] * h1.w;
       }
     }
   }
+  // one reduce-scatter for all of them (the same pairwise sums as a butterfly per value): lane
+  // group v >> log2 holds (row k, sequence b) and its first lane writes it
+  const float a = ReduceScatter<kV, 16>::run(acc);
+  constexpr int kSh = 5 - ilog2(kV);
+  const int v = lane >> kSh, k = v / KB, b = v % KB;
+  float ub = 0.f;
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
-    const int row = row0 + k * stride;
-#pragma unroll
-    for (int b = 0; b < KB; ++b) {
-      if (b < B) {
-        const float a = warp_sum(acc[k][b]);
-        const float ub = __shfl_sync(0xffffffffu, uhb[k], b);
-        if (lane == 0 && row < rows) {
-          if (row < R) {
-            const float x = a + ub;
-            p.u[static_cast<size_t>(b) * R + row] = x / (1.f + expf(-x));
-          } else {
-            gh[static_cast<size_t>(b) * 3 * Ds + row - R] = a;
-          }
-        }
-      }
+  for (int i = 0; i < NR; ++i) {
+    const float t = __shfl_sync(0xffffffffu, uhb[i], b);
+    if (i == k) ub = t;
+  }
+  const int row = row0 + k * stride;
+  if ((lane & ((1 << kSh) - 1)) == 0 && k < NR && b < B && row < rows) {
+    if (row < R) {
+      const float x = a + ub;
+      p.u[static_cast<size_t>(b) * R + row] = x / (1.f + expf(-x));
+    } else {
+      gh[static_cast<size_t>(b) * 3 * Ds + row - R] = a;
     }
-    if (count_u && lane == 0 && row < R)  // this row of u_j is written for every sequence
+  }
+  if (count_u) {  // the rows of u_j among these are written for every sequence
+    __syncwarp();
+    if (lane < NR && row0 + lane * stride < min(R, rows))
       asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.ucount) : "memory");
   }
 }
 
 template <int KB>
-__device__ __forceinline__ void ub_phase(const RolloutParams& p, int j, const float* s_h, int gw, int nwarps,
+__device__ __forceinline__ void ub_phase(const RolloutParams& p, int j, const float* s_h, int hs, int gw, int nwarps,
                                          int lane, uint64_t pol) {
   const int R = p.R;
   const int rows = R + (j + 1 < p.K ? 3 * p.Ds : 0);
@@ -623,16 +684,16 @@ __device__ __forceinline__ void ub_phase(const RolloutParams& p, int j, const fl
       // thread counts their nu rows (one atomic per CTA rather than per row)
       const int warp = gw - static_cast<int>(blockIdx.x) * kRollWarps;
       const int nu = min(kRollWarps, R - static_cast<int>(blockIdx.x) * kRollWarps);
-      ub_rows<KB, 1>(p, j, s_h, gw, 0, R, lane, pol, false);
+      ub_rows<KB, 1>(p, j, s_h, hs, gw, 0, R, lane, pol, false);
       asm volatile("bar.sync 2, %0;" ::"r"(nu * 32) : "memory");
       if (warp == 0 && lane == 0)
         asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.ucount), "r"(static_cast<unsigned>(nu)) : "memory");
     } else {
       const int n = nwarps - R;
-      for (int row0 = gw; row0 < rows; row0 += 4 * n) ub_rows<KB, 4>(p, j, s_h, row0, n, rows, lane, pol);
+      for (int row0 = gw; row0 < rows; row0 += 4 * n) ub_rows<KB, 4>(p, j, s_h, hs, row0, n, rows, lane, pol);
     }
   } else {
-    for (int row0 = gw; row0 < rows; row0 += 3 * nwarps) ub_rows<KB, 3>(p, j, s_h, row0, nwarps, rows, lane, pol);
+    for (int row0 = gw; row0 < rows; row0 += 3 * nwarps) ub_rows<KB, 3>(p, j, s_h, hs, row0, nwarps, rows, lane, pol);
   }
 }
 
@@ -880,25 +941,41 @@ __device__ void sample_step(const RolloutParams& p, int j, const float4 (&mine)[
   compute_sync();
 }
 
+// This CTA's rows of step j's base logits, copied asynchronously into shared memory; 16 bytes at a time
+// where the rows' alignment allows it (B = 4: 4 copies a thread instead of 16).
+__device__ __forceinline__ void copy_base(const RolloutParams& p, int j, float* s_base, int r_lo, int r_n, int rows_cta) {
+  const int B = p.B, K = p.K, V = p.V;
+  const bool vec = ((V | rows_cta) & 3) == 0 && ((reinterpret_cast<uintptr_t>(p.base) | smem_u32(s_base)) & 15u) == 0;
+  for (int b = 0; b < B; ++b) {
+    const float* src = p.base + (static_cast<size_t>(b) * K + j) * V + r_lo;
+    float* dst = s_base + b * rows_cta;
+    if (vec) {
+      for (int r = threadIdx.x * 4; r < r_n; r += 4 * kRollThreads) cp_async16(dst + r, src + r);
+    } else {
+      for (int r = threadIdx.x; r < r_n; r += kRollThreads) cp_async4(dst + r, src + r);
+    }
+  }
+}
+
 // Greedy end of step j (p.best set): the CTA's best row of each sequence as one key -- the step
 // (so that no earlier step's key competes), the logit in order-preserving form, then the id
 // inverted, so that the largest key over the CTAs is the step's maximum with ties to the lowest
-// id (ids below 2^22) -- from two integer warp reductions per warp; thread 0 folds the warps'
-// keys into the sequence's slot with one red.max and arrives at the grid barrier.  While the
-// other CTAs arrive (before the arrival at the last step, which no later barrier follows), each
-// warp reduces its (max, sum of exp) of every sequence and writes it to the step's partials (the
-// log-probabilities are merged from them once, after the last step: greedy_logp); then thread 0
-// reads the slot.  The slots alternate by step parity: a CTA
-// updates step j + 2's only after every CTA has passed step j + 1's barrier, so after every read
-// of step j's.  Returns false if the barrier gave up.
+// id (ids below 2^22) -- from two integer warp reductions per warp; lane b of warp 0 folds the
+// warps' keys of sequence b into its slot with one red.max, and lane 0 arrives at the grid barrier.
+// While the other CTAs arrive (before the arrival at the last step, which no later barrier
+// follows), each warp reduces its (max, sum of exp) of every sequence and writes it to the step's
+// partials (the log-probabilities are merged from them once, after the last step: greedy_logp);
+// then lane b reads slot b.  The slots alternate by step parity: a CTA updates step j + 2's only
+// after every CTA has passed step j + 1's barrier, so after every read of step j's.  Returns false
+// if the barrier gave up.
 // kRace (the exponential race, the seeded sampled loop): the keys are those of the perturbed logits
 // (`pick`), and each warp's partial also carries its pick's id and logit, from which greedy_logp
 // takes the drawn token's logit.
-// s_base_next (the resident kernel): the next step's base logits are copied into it (cp.async)
+// copy_next (the resident kernel): the next step's base logits are copied into s_base (cp.async)
 // while the barrier completes.
 template <int KB, bool kRace>
 __device__ bool finish_greedy(const RolloutParams& p, int j, Lse (&st)[KB], const Pick (&pick)[KB], int* s_tok,
-                              unsigned& nbar, volatile int* s_fail, float* s_base_next, int r_lo, int r_n,
+                              unsigned& nbar, volatile int* s_fail, bool copy_next, float* s_base, int r_lo, int r_n,
                               int rows_cta) {
   __shared__ unsigned long long s_key[kRollWarps][kRollMaxB];
   __shared__ int s_go;
@@ -927,29 +1004,20 @@ __device__ bool finish_greedy(const RolloutParams& p, int j, Lse (&st)[KB], cons
       }
     }
   }
-  // each warp's (max, sum of exp) of every sequence, for the log-probabilities
+  // each warp's (max, sum of exp) of every sequence, for the log-probabilities: the maximum from one
+  // integer reduction, then the lanes' sums rescaled to it once and added
   float4* part = reinterpret_cast<float4*>(p.partials) +
                  (static_cast<size_t>(j) * grid + blockIdx.x) * kRollWarps * kRollMaxB;
   auto write_partials = [&]() {
 #pragma unroll
     for (int b = 0; b < KB; ++b) {
       if (b < B) {
-        Lse a = st[b];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-          Lse t;
-          t.m = __shfl_xor_sync(0xffffffffu, a.m, o);
-          t.s = __shfl_xor_sync(0xffffffffu, a.s, o);
-          t.i = __shfl_xor_sync(0xffffffffu, a.i, o);
-          lse_merge(a, t);
-        }
+        const uint32_t mo = kRace ? __reduce_max_sync(0xffffffffu, f32_ord(st[b].m)) : whi[b];
+        const float m = (kRace || mo != 0u) ? f32_unord(mo) : -INFINITY;
+        const float sum = warp_sum(lse_scaled(st[b], m));
         if (lane == 0) {
-          if constexpr (kRace) {
-            const int pid = whi[b] != 0u ? static_cast<int>(kGreedyIdMask - wlo[b]) : -1;
-            part[warp * kRollMaxB + b] = make_float4(a.m, a.s, __int_as_float(pid), wraw[b]);
-          } else {
-            part[warp * kRollMaxB + b] = make_float4(a.m, a.s, __int_as_float(a.i), 0.f);
-          }
+          const int id = whi[b] != 0u ? static_cast<int>(kGreedyIdMask - wlo[b]) : -1;
+          part[warp * kRollMaxB + b] = make_float4(m, sum, __int_as_float(id), wraw[b]);
         }
       }
     }
@@ -967,46 +1035,46 @@ __device__ bool finish_greedy(const RolloutParams& p, int j, Lse (&st)[KB], cons
                                     : 0ull;
   }
   compute_sync();
-  if (tid == 0) {
-    for (int b = 0; b < B; ++b) {
+  if (warp == 0) {
+    if (lane < B) {
       unsigned long long k = 0ull;
-      for (int w = 0; w < kRollWarps; ++w) k = s_key[w][b] > k ? s_key[w][b] : k;
-      if (k != 0ull) asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(slot + b), "l"(k) : "memory");
+#pragma unroll
+      for (int w = 0; w < kRollWarps; ++w) k = s_key[w][lane] > k ? s_key[w][lane] : k;
+      if (k != 0ull) asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(slot + lane), "l"(k) : "memory");
     }
+    __syncwarp();
     // release at GPU scope: this CTA's keys (and its earlier writes) before its arrival
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.barrier) : "memory");
+    if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.barrier) : "memory");
   }
-  if (s_base_next != nullptr && j + 1 < K) {  // phase C has read this step's
-    for (int e = tid; e < B * r_n; e += kRollThreads) {
-      const int b = e / r_n, r = e - b * r_n;
-      cp_async4(s_base_next + b * rows_cta + r, p.base + (static_cast<size_t>(b) * K + j + 1) * p.V + r_lo + r);
-    }
-  }
+  if (copy_next && !last) copy_base(p, j + 1, s_base, r_lo, r_n, rows_cta);  // phase C has read this step's
   if (!last) write_partials();
-  if (tid == 0) {
-    const unsigned target = (nbar + 1) * static_cast<unsigned>(grid);
-    const long long t0 = clock64();
-    while (true) {
-      unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.barrier) : "memory");
-      if (v >= target) break;
-      if (clock64() - t0 > kWaitCycles) {
-        set_status(p.status, kStatusTimeout);
-        *s_fail = 1;
-        break;
+  if (warp == 0) {
+    int go = 0;
+    if (lane == 0) {
+      const unsigned target = (nbar + 1) * static_cast<unsigned>(grid);
+      const long long t0 = clock64();
+      while (true) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.barrier) : "memory");
+        if (v >= target) break;
+        if (clock64() - t0 > kWaitCycles) {
+          set_status(p.status, kStatusTimeout);
+          *s_fail = 1;
+          break;
+        }
+        __nanosleep(32);
       }
-      __nanosleep(32);
+      go = *s_fail == 0;
+      s_go = go;
     }
-    s_go = *s_fail == 0;
-    if (s_go) {  // every CTA's red.max came before its arrival
-      for (int b = 0; b < B; ++b) {
-        const unsigned long long key = __ldcg(slot + b);
-        const int tok = static_cast<int>(key >> 54) == j + 1
-                            ? static_cast<int>(kGreedyIdMask - static_cast<unsigned>(key & kGreedyIdMask))
-                            : 0;  // no row with a finite logit anywhere
-        s_tok[b] = tok;
-        if (blockIdx.x == 0) p.tokens[static_cast<size_t>(b) * K + j] = tok;
-      }
+    go = __shfl_sync(0xffffffffu, go, 0);  // lane 0's acquire orders the other lanes' reads
+    if (go && lane < B) {                  // every CTA's red.max came before its arrival
+      const unsigned long long key = __ldcg(slot + lane);
+      const int tok = static_cast<int>(key >> 54) == j + 1
+                          ? static_cast<int>(kGreedyIdMask - static_cast<unsigned>(key & kGreedyIdMask))
+                          : 0;  // no row with a finite logit anywhere
+      s_tok[lane] = tok;
+      if (blockIdx.x == 0) p.tokens[static_cast<size_t>(lane) * K + j] = tok;
     }
   }
   ++nbar;
@@ -1027,8 +1095,8 @@ __device__ __forceinline__ bool finish_step(const RolloutParams& p, int j, Lse (
   const int B = p.B, V = p.V, tid = threadIdx.x;
   const int grid = static_cast<int>(gridDim.x);
   if (kRace || p.best != nullptr)
-    return finish_greedy<KB, kRace>(p, j, st, pick, s_tok, nbar, s_fail, (resident && p.fast_gates) ? s_logit : nullptr,
-                                r_lo, r_n, rows_cta);
+    return finish_greedy<KB, kRace>(p, j, st, pick, s_tok, nbar, s_fail, resident && p.fast_gates, s_logit, r_lo, r_n,
+                                    rows_cta);
   float4* part = reinterpret_cast<float4*>(p.partials) + static_cast<size_t>(j & 1) * grid * kRollMaxB;
   block_reduce(st, s_red, B);  // ends with a barrier: every row's final logit is in s_logit
   if (tid < B) {
@@ -1077,51 +1145,41 @@ __device__ __forceinline__ bool finish_step(const RolloutParams& p, int j, Lse (
 
 // Greedy mode, after the last step: the log-probability of each step's token.  The token is the
 // step's argmax, so its log-softmax is -log of the sum of exp(L - max) over the vocabulary, the
-// merge of every warp's partials of that step (CTA c takes steps c, c + grid, ...).  Called by
-// the compute threads of every CTA after the last step's barrier: every step's partials were
-// written before some later arrival at a grid barrier (the last step's before its own).
+// merge of every warp's partials of that step (CTA c takes the (step, sequence) pairs c, c + grid,
+// ...).  Called by the compute threads of every CTA after the last step's barrier: every step's
+// partials were written before some later arrival at a grid barrier (the last step's before its own).
 // kRace: the token is the perturbed maximum, so its log-softmax is its logit - max - log(sum); the
 // logit is the one the warp whose pick was the token wrote with its partial.  The token of a
 // step before the last is read from the outputs (CTA 0 wrote it before its next arrival); the
 // last step's is s_tok, which every CTA holds.
-template <int KB, bool kRace>
+template <bool kRace>
 __device__ void greedy_logp(const RolloutParams& p, Lse (*s_red)[kRollMaxB], const int* s_tok) {
-  __shared__ float s_raw[kRollMaxB];
-  const int B = p.B, K = p.K, tid = threadIdx.x;
+  __shared__ float s_raw;
+  const int K = p.K, tid = threadIdx.x;
   const int grid = static_cast<int>(gridDim.x);
   const int nw = grid * kRollWarps;
-  for (int j = blockIdx.x; j < K; j += grid) {
-    const float4* part = reinterpret_cast<const float4*>(p.partials) + static_cast<size_t>(j) * nw * kRollMaxB;
-    int tok[KB];
-#pragma unroll
-    for (int b = 0; b < KB; ++b) {
-      tok[b] = -2;
-      if (kRace && b < B) tok[b] = j + 1 == K ? s_tok[b] : __ldcg(p.tokens + static_cast<size_t>(b) * K + j);
-    }
-    if (kRace && tid < B) s_raw[tid] = 0.f;
+  for (int i = blockIdx.x; i < K * p.B; i += grid) {
+    const int j = i % K, b = i / K;
+    const float4* part = reinterpret_cast<const float4*>(p.partials) + static_cast<size_t>(j) * nw * kRollMaxB + b;
+    int tok = -2;
+    if (kRace) tok = j + 1 == K ? s_tok[b] : __ldcg(p.tokens + static_cast<size_t>(b) * K + j);
+    if (kRace && tid == 0) s_raw = 0.f;
     compute_sync();
-    Lse st[KB];
-#pragma unroll
-    for (int b = 0; b < KB; ++b) st[b] = lse_empty();
+    Lse st[1] = {lse_empty()};
     for (int c = tid; c < nw; c += kRollThreads) {
-#pragma unroll
-      for (int b = 0; b < KB; ++b) {
-        if (b < B) {
-          const float4 f = __ldcg(part + static_cast<size_t>(c) * kRollMaxB + b);
-          Lse t;
-          t.m = f.x; t.s = f.y; t.i = __float_as_int(f.z);
-          lse_merge(st[b], t);
-          if (kRace && __float_as_int(f.z) == tok[b]) s_raw[b] = f.w;  // the one warp that held the token
-        }
-      }
+      const float4 f = __ldcg(part + static_cast<size_t>(c) * kRollMaxB);
+      Lse t;
+      t.m = f.x; t.s = f.y; t.i = __float_as_int(f.z);
+      lse_merge(st[0], t);
+      if (kRace && __float_as_int(f.z) == tok) s_raw = f.w;  // the one warp that held the token
     }
-    block_reduce(st, s_red, B);
-    if (tid < B) {
-      Lse a = s_red[0][tid];
-      for (int w = 1; w < kRollWarps; ++w) lse_merge(a, s_red[w][tid]);
-      p.logp[static_cast<size_t>(tid) * K + j] = kRace ? s_raw[tid] - a.m - logf(a.s) : -logf(a.s);
+    block_reduce(st, s_red, 1);
+    if (tid == 0) {
+      Lse a = s_red[0][0];
+      for (int w = 1; w < kRollWarps; ++w) lse_merge(a, s_red[w][0]);
+      p.logp[static_cast<size_t>(b) * K + j] = kRace ? s_raw - a.m - logf(a.s) : -logf(a.s);
     }
-    compute_sync();  // s_red is read before the next step's reduction overwrites it
+    compute_sync();  // s_red is read before the next pair's reduction overwrites it
   }
 }
 
@@ -1195,31 +1253,143 @@ __device__ __forceinline__ float lane_gumbel(unsigned long long seed, int lane, 
 // Phase C on the tensor cores (kMma).  A CTA's W2 rows form 128-row blocks: the first mma_tb in
 // tensor memory as the MMA's A operand (row in lane, K along the columns), the next mma_sb in
 // shared memory as 128-byte swizzled K-major tiles (loaded once by TMA); rows past those blocks
-// are read through L2 on the CUDA cores as in the other layout.  u_j is the B operand with
-// N = 16 rows: row 2b holds bf16(u_j[b]) and row 2b + 1 the bf16 of what that rounding left out,
-// so that D[:, 2b] + D[:, 2b + 1] is W2 u_j to about 2^-16 relative (fp32 accumulation, the
-// precision the CUDA-core layout keeps u in).  Each block's MMAs go into its own 16 columns of D,
-// issued by one thread of its own warp; the epilogue adds the staged base logit and b2 of each row.
+// are read through L2 (RestTile; inverse CDF: on the CUDA cores).  u_j is the B operand: rows
+// 3b, 3b + 1 and 3b + 2 hold bf16 terms of u_j[b] that add up to it (u_terms), so that
+// D[:, 3b] + (D[:, 3b + 1] + D[:, 3b + 2]) is W2 u_j with u kept to fp32's 24 bits (three terms; two,
+// 16 bits, under the inverse-CDF rule), accumulated in fp32.  Each block's MMAs go into its own kN columns of D (16, or 32 above
+// four sequences), issued by one thread of its own warp; the epilogue adds the staged base logit and
+// b2 of each row.
 // Tensor memory (512 columns): A block i at columns [i r/2, (i+1) r/2), D of block i at
-// mma_tb r/2 + 16 i.  Shared memory from a 1024-byte boundary: the A blocks (r/64 tiles of
-// 128 rows x 64 columns each), the B operand (r/64 tiles of 16 rows x 64 columns), then u, the
+// mma_tb r/2 + kN i.  Shared memory from a 1024-byte boundary: the A blocks (r/64 tiles of
+// 128 rows x 64 columns each), the B operand (r/64 tiles of kN rows x 64 columns), then u, the
 // base logits, b2 and h as in the other layout.
-constexpr int kMmaBopTileBytes = 16 * 128;   // B operand: 16 rows x 64 bf16 columns
+__host__ __device__ constexpr int mma_n(int B) { return B <= 4 ? 16 : 32; }  // rows of the B operand
 constexpr int kMmaTileBytes = 128 * 128;     // A block: 128 rows x 64 bf16 columns
-constexpr int kMmaMaxL2Rows = 384;           // at most this many rows a CTA reads through L2
+constexpr int kMmaMaxL2Rows = 384;           // inverse CDF: at most this many rows a CTA reads through L2
 
 // Byte offset of element (n, k) of the B operand in its 128-byte swizzled K-major tiles: tile
-// k / 64, 8-row groups 1024 bytes apart, 16-byte chunk c of row r stored at chunk c ^ (r % 8).
-__device__ __forceinline__ uint32_t bop_offset(int n, int k) {
+// k / 64 (tile_bytes each), 8-row groups 1024 bytes apart, 16-byte chunk c of row r stored at
+// chunk c ^ (r % 8).
+__device__ __forceinline__ uint32_t bop_offset(int n, int k, int tile_bytes) {
   const int kin = k & 63, r = n & 7;
-  return static_cast<uint32_t>((k >> 6) * kMmaBopTileBytes + (n >> 3) * 1024 + r * 128 + (((kin >> 3) ^ r) << 4) +
+  return static_cast<uint32_t>((k >> 6) * tile_bytes + (n >> 3) * 1024 + r * 128 + (((kin >> 3) ^ r) << 4) +
                                (kin & 7) * 2);
 }
 
-template <int KB, bool kMma, bool kRace>
+// The bf16 terms of v: v rounded, what that leaves rounded, and (three) what both leave, which
+// is exact: 8 + 8 + 8 bits.  Non-finite values are their first term; a finite v past bf16's
+// largest is truncated to it.  Two terms: the third is zero.
+__device__ __forceinline__ void u_terms(float v, int terms, __nv_bfloat16 (&t)[3]) {
+  t[0] = __float2bfloat16_rn(v);
+  if (isinf(__bfloat162float(t[0])) && !isinf(v)) t[0] = __float2bfloat16_rz(v);
+  const float hi = __bfloat162float(t[0]);
+  const float r1 = isfinite(hi) ? v - hi : 0.f;
+  t[1] = __float2bfloat16_rn(r1);
+  t[2] = __float2bfloat16_rn(terms > 2 ? r1 - __bfloat162float(t[1]) : 0.f);
+}
+
+// The first 3 KB accumulator columns (one row's dot products) from a D block's column address.
+template <int KB>
+__device__ __forceinline__ void ld_acc(uint32_t taddr, float (&d)[KB == 1 ? 4 : KB == 2 ? 8 : KB == 4 ? 16 : 32]) {
+  if constexpr (KB == 1) tc_ld_x4(taddr, d);
+  else if constexpr (KB == 2) tc_ld_x8(taddr, d);
+  else if constexpr (KB == 4) tc_ld_x16(taddr, d);
+  else tc_ld_x32(taddr, d);
+}
+
+// The rows past the MMA blocks (kMma, greedy and race): 16-row tiles on mma.sync, a warp's tiles
+// read through L2 straight into A fragments.  In each 64-column chunk lane 4 g + t loads columns
+// 16 t .. 16 t + 15 of rows g and g + 8 (32 contiguous bytes a row) and MMA step s of the chunk takes
+// words 2 s and 2 s + 1 of those; B's column g is read the same way from the swizzled B operand, so
+// both sides meet at the same columns.  Bound by L2 (512 bytes a row at about 29 B a clock and SM):
+// the first tile's loads are issued before the wait for u_j, whose latency they share.  The CUDA-core
+// form took 3.6 us a step for 232 rows at B = 1 and 8.4 us for 360 rows at B = 4.
+template <int KB>
+struct RestTile {
+  static constexpr int kNt = KB <= 2 ? 1 : KB == 4 ? 2 : 3;  // 8-column B tiles
+  static constexpr int kSeq = KB == 8 ? 2 : 1;               // sequences a lane ends with: t (and t + 4)
+  uint4 a[4][4];                                             // [64-column chunk][row g lo, hi, row g + 8 lo, hi]
+
+  // Row of the B operand that column n of tile nt holds (term i of sequence b is row 3 b + i).
+  // Pairs of columns 2 t, 2 t + 1 end in lane t: the first two terms of sequence t; the third terms
+  // go to lane 2 (KB <= 2: columns 4 + t), to the even columns of the second tile (KB = 4), or to
+  // the third tile (KB = 8: sequence t even, t + 4 odd).  The last row of the operand is zero.
+  static __device__ __forceinline__ int b_row(int nt, int n) {
+    constexpr int kZero = mma_n(KB) - 1;
+    const int t = n >> 1, odd = n & 1;
+    if (KB <= 2) return n < 4 ? 3 * t + odd : n < 6 ? 3 * (n - 4) + 2 : kZero;
+    if (KB == 4) return nt == 0 ? 3 * t + odd : odd ? kZero : 3 * t + 2;
+    return nt < 2 ? 3 * (t + 4 * nt) + odd : 3 * (t + 4 * odd) + 2;
+  }
+
+  __device__ __forceinline__ void load(const __nv_bfloat16* w2, int R, int nrows, int lane, uint64_t pol) {
+    const int g = lane >> 2, t = lane & 3;
+    const __nv_bfloat16* ra = w2 + static_cast<size_t>(g) * R + 16 * t;
+    const bool va = g < nrows, vb = g + 8 < nrows;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const bool in = 64 * c < R;
+      a[c][0] = in && va ? ld16_hint(ra + 64 * c, pol) : make_uint4(0, 0, 0, 0);
+      a[c][1] = in && va ? ld16_hint(ra + 64 * c + 8, pol) : make_uint4(0, 0, 0, 0);
+      a[c][2] = in && vb ? ld16_hint(ra + 8 * R + 64 * c, pol) : make_uint4(0, 0, 0, 0);
+      a[c][3] = in && vb ? ld16_hint(ra + 8 * R + 64 * c + 8, pol) : make_uint4(0, 0, 0, 0);
+    }
+  }
+
+  // d[h][i]: W2 u of row g + 8 h and sequence t + 4 i.
+  __device__ __forceinline__ void multiply(const uint8_t* s_bop, int R, int lane, float (&d)[2][kSeq]) const {
+    const int g = lane >> 2, t = lane & 3;
+    float acc[kNt][4];
+#pragma unroll
+    for (int nt = 0; nt < kNt; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (64 * c >= R) break;
+      const uint32_t x[4][4] = {{a[c][0].x, a[c][0].y, a[c][0].z, a[c][0].w}, {a[c][1].x, a[c][1].y, a[c][1].z, a[c][1].w},
+                                {a[c][2].x, a[c][2].y, a[c][2].z, a[c][2].w}, {a[c][3].x, a[c][3].y, a[c][3].z, a[c][3].w}};
+#pragma unroll
+      for (int nt = 0; nt < kNt; ++nt) {
+        const int n = b_row(nt, g), r = n & 7;
+        const uint8_t* row = s_bop + c * (mma_n(KB) * 128) + (n >> 3) * 1024 + r * 128;
+        const uint4 b0 = *reinterpret_cast<const uint4*>(row + (((2 * t) ^ r) << 4));
+        const uint4 b1 = *reinterpret_cast<const uint4*>(row + (((2 * t + 1) ^ r) << 4));
+        const uint32_t y[2][4] = {{b0.x, b0.y, b0.z, b0.w}, {b1.x, b1.y, b1.z, b1.w}};
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const uint32_t am[4] = {x[s >> 1][2 * (s & 1)], x[2 + (s >> 1)][2 * (s & 1)], x[s >> 1][2 * (s & 1) + 1],
+                                  x[2 + (s >> 1)][2 * (s & 1) + 1]};
+          const uint32_t bm[2] = {y[s >> 1][2 * (s & 1)], y[s >> 1][2 * (s & 1) + 1]};
+          mma_sync_16816(acc[nt], am, bm);
+        }
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if constexpr (KB <= 2) {
+        const float x0 = __shfl_sync(0xffffffffu, acc[0][2 * h], (lane & ~3) | 2);
+        const float x1 = __shfl_sync(0xffffffffu, acc[0][2 * h + 1], (lane & ~3) | 2);
+        d[h][0] = acc[0][2 * h] + (acc[0][2 * h + 1] + (t == 0 ? x0 : x1));
+      } else if constexpr (KB == 4) {
+        d[h][0] = acc[0][2 * h] + (acc[0][2 * h + 1] + acc[1][2 * h]);
+      } else {
+        d[h][0] = acc[0][2 * h] + (acc[0][2 * h + 1] + acc[2][2 * h]);
+        d[h][1] = acc[1][2 * h] + (acc[1][2 * h + 1] + acc[2][2 * h + 1]);
+      }
+    }
+  }
+};
+
+// kCdf (kMma only): the inverse-CDF rule, whose rows past the MMA blocks stay on the CUDA cores and
+// whose sums keep their order, since they decide the draws.
+template <int KB, bool kMma, bool kRace, bool kCdf>
 __global__ void __launch_bounds__(kRollThreads, 1)
     rollout_resident_kernel(const RolloutParams p, const __grid_constant__ CUtensorMap tm_w2) {
-  static_assert(!kMma || KB <= 2, "the B operand holds two rows per sequence in its 16");
+  constexpr int kN = mma_n(KB);            // columns of D, rows of the B operand
+  constexpr int kBopTileBytes = kN * 128;  // B operand: kN rows x 64 bf16 columns
+  static_assert(3 * KB < kN, "the B operand holds three rows per sequence and a zero row");
+  static_assert(!kCdf || (kMma && !kRace && KB <= 2), "the inverse-CDF form of the tensor-core layout");
+  constexpr bool kRest = kMma && !kCdf;  // rows past the MMA blocks on mma.sync
+  const int hs = (p.Ds + 255) & ~255;    // stride of a sequence's h in shared memory (h_slot)
   const int B = p.B, K = p.K, V = p.V, R = p.R;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nwarps = gridDim.x * kRollWarps;
@@ -1239,7 +1409,7 @@ __global__ void __launch_bounds__(kRollThreads, 1)
                        : s_dyn;
   uint8_t* s_bop = s_al + static_cast<size_t>(kMma ? p.mma_sb : 0) * (R / 64) * kMmaTileBytes;  // kMma
   __nv_bfloat16* s_w2 = reinterpret_cast<__nv_bfloat16*>(s_dyn);  // [smem_rows][R] (!kMma)
-  float* s_u = kMma ? reinterpret_cast<float*>(s_bop + (R / 64) * kMmaBopTileBytes)
+  float* s_u = kMma ? reinterpret_cast<float*>(s_bop + (R / 64) * kBopTileBytes)
                     : reinterpret_cast<float*>(s_dyn + static_cast<size_t>(p.smem_rows) * R * 2);  // [B][R]
   float* s_base = s_u + B * R;                                                          // [B][rows_cta]
   float* s_b2 = s_base + B * rows_cta;                                                  // [rows_cta]
@@ -1331,8 +1501,8 @@ __global__ void __launch_bounds__(kRollThreads, 1)
           tc_st_x16(tq + static_cast<uint32_t>(i * cols + half * hc + c0), r);
         }
       }
-      // the B operand's rows 2B .. 15 stay zero
-      for (int e = tid; e < (R / 64) * kMmaBopTileBytes / 16; e += kRollThreads)
+      // the B operand's rows past 3 B stay zero
+      for (int e = tid; e < (R / 64) * kBopTileBytes / 16; e += kRollThreads)
         reinterpret_cast<uint4*>(s_bop)[e] = make_uint4(0, 0, 0, 0);
     } else {
       // ---- fill: tensor-memory rows.  Warp w writes lane quarter q = w % 4, rows 64 (w / 4) ..
@@ -1371,33 +1541,41 @@ __global__ void __launch_bounds__(kRollThreads, 1)
       // this step's base logits for the CTA's rows: asynchronous copies that land during A and B
       // (greedy two-barrier step: issued by the previous step's finish, from step 1 on)
       if (j == 0 || p.best == nullptr || !p.fast_gates) {
-        for (int e = tid; e < B * r_n; e += kRollThreads) {
-          const int b = e / r_n, r = e - b * r_n;
-          cp_async4(s_base + b * rows_cta + r, p.base + (static_cast<size_t>(b) * K + j) * V + r_lo + r);
-        }
+        copy_base(p, j, s_base, r_lo, r_n, rows_cta);
       }
+      [[maybe_unused]] RestTile<KB> rest;  // kRest: this warp's tile of the rows past the MMA blocks
+      [[maybe_unused]] const __nv_bfloat16* w2_rest = p.w2 + static_cast<size_t>(r_lo + n_t + n_s) * R;
       if (p.fast_gates) {
-        gates_all(p, j, s_tok, s_h);
+        gates_all<KB>(p, j, s_tok, s_h, hs);
         compute_sync();  // h_j of every sequence in this CTA's shared memory
-        ub_phase<KB>(p, j, s_h, gw, nwarps, lane, pol_ab);
+        ub_phase<KB>(p, j, s_h, hs, gw, nwarps, lane, pol_ab);
+        if constexpr (kRest) rest.load(w2_rest + static_cast<size_t>(16 * warp) * R, R, n_g - 16 * warp, lane, pol_rest);
         // phase C needs u_j only: every one of its R rows counted, not a grid barrier
         if (!wait_count(p.ucount, static_cast<unsigned>(R) * (j + 1), p.status, &s_fail)) break;
       } else {
         gru_phase(p, s_tok, hprev, hcur, gw, nwarps, lane, pol_ab);
         if (!grid_barrier(p.barrier, nbar++, p.status, &s_fail)) break;
         u_phase(p, j, hcur, gw, nwarps, lane, pol_ab);
+        if constexpr (kRest) rest.load(w2_rest + static_cast<size_t>(16 * warp) * R, R, n_g - 16 * warp, lane, pol_rest);
         if (!grid_barrier(p.barrier, nbar++, p.status, &s_fail)) break;
       }
-      for (int e = tid; e < B * R; e += kRollThreads) {
-        const float v = __ldcg(p.u + e);
-        s_u[e] = v;
-        if constexpr (kMma) {  // u_j as the B operand: rows 2b (bf16 of u) and 2b + 1 (the rest)
+      if constexpr (kMma) {  // u_j as the B operand: rows 3b .. 3b + 2, four columns at a time (r % 64 == 0)
+        for (int e = 4 * tid; e < B * R; e += 4 * kRollThreads) {
+          const float4 v4 = __ldcg(reinterpret_cast<const float4*>(p.u + e));
+          if constexpr (kCdf) *reinterpret_cast<float4*>(s_u + e) = v4;  // the CUDA-core rows' operand
+          const float v[4] = {v4.x, v4.y, v4.z, v4.w};
           const int b = e / R, k = e - b * R;
-          const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-          const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-          *reinterpret_cast<__nv_bfloat16*>(s_bop + bop_offset(2 * b, k)) = hi;
-          *reinterpret_cast<__nv_bfloat16*>(s_bop + bop_offset(2 * b + 1, k)) = lo;
+          __nv_bfloat16 t[4][3];
+#pragma unroll
+          for (int q4 = 0; q4 < 4; ++q4) u_terms(v[q4], kCdf ? 2 : 3, t[q4]);
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            __nv_bfloat162 w[2] = {__halves2bfloat162(t[0][i], t[1][i]), __halves2bfloat162(t[2][i], t[3][i])};
+            *reinterpret_cast<uint2*>(s_bop + bop_offset(3 * b + i, k, kBopTileBytes)) = *reinterpret_cast<uint2*>(w);
+          }
         }
+      } else {
+        for (int e = tid; e < B * R; e += kRollThreads) s_u[e] = __ldcg(p.u + e);
       }
       if constexpr (kMma) {
         fence_proxy_async_smem();  // the B operand, for the tensor core
@@ -1414,18 +1592,18 @@ __global__ void __launch_bounds__(kRollThreads, 1)
           if (j == 0 && fill_any) ok = mbar_wait(&s_fill, 0, &s_fail, p.status);
           if (ok) {
             tc_fence_after();
-            constexpr uint32_t kIdesc = idesc_bf16_f32(128, 16);
+            constexpr uint32_t kIdesc = idesc_bf16_f32(128, kN);
             const uint64_t bd0 = smem_desc_sw128(smem_u32(s_bop));
             const uint32_t ab_a = smem_u32(s_al);
             const int ksteps = R / 16;
             for (int i = kRollWarps - 1 - warp; i < n_blk; i += kRollWarps) {
-              const uint32_t d = tbase + static_cast<uint32_t>(dcol0 + 16 * i);
+              const uint32_t d = tbase + static_cast<uint32_t>(dcol0 + kN * i);
               if (i < p.mma_tb) {
                 const uint32_t a0 = tbase + static_cast<uint32_t>(i * (R / 2));
 #pragma unroll 4
                 for (int kk = 0; kk < ksteps; ++kk)
                   tc_mma_bf16_ta(d, a0 + static_cast<uint32_t>(8 * kk),
-                                 bd0 + static_cast<uint64_t>((kk >> 2) * (kMmaBopTileBytes >> 4) + 2 * (kk & 3)), kIdesc,
+                                 bd0 + static_cast<uint64_t>((kk >> 2) * (kBopTileBytes >> 4) + 2 * (kk & 3)), kIdesc,
                                  kk > 0 ? 1u : 0u);
               } else {
                 const uint64_t ad0 =
@@ -1433,7 +1611,7 @@ __global__ void __launch_bounds__(kRollThreads, 1)
 #pragma unroll 4
                 for (int kk = 0; kk < ksteps; ++kk)
                   tc_mma_bf16(d, ad0 + static_cast<uint64_t>((kk >> 2) * (kMmaTileBytes >> 4) + 2 * (kk & 3)),
-                              bd0 + static_cast<uint64_t>((kk >> 2) * (kMmaBopTileBytes >> 4) + 2 * (kk & 3)), kIdesc,
+                              bd0 + static_cast<uint64_t>((kk >> 2) * (kBopTileBytes >> 4) + 2 * (kk & 3)), kIdesc,
                               kk > 0 ? 1u : 0u);
               }
             }
@@ -1444,13 +1622,23 @@ __global__ void __launch_bounds__(kRollThreads, 1)
         }
         if (tid == 0) ++mma_steps;
       }
-      float ur[KB][8];  // u at this lane's 8 columns (zero past r)
-#pragma unroll
-      for (int b = 0; b < KB; ++b)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) ur[b][e] = (b < B && lane * 8 < R) ? s_u[(b < B && lane * 8 < R) ? b * R + lane * 8 + e : 0] : 0.f;
       Lse mine = lse_empty();
       Pick pmine = pick_empty();  // kRace: the perturbed maximum of the same rows
+      Lse st[KB];
+      Pick pst[KB];
+#pragma unroll
+      for (int b = 0; b < KB; ++b) {
+        st[b] = lse_empty();
+        pst[b] = pick_empty();
+      }
+      float ur[KB][8];  // CUDA-core rows: u at this lane's 8 columns (zero past r)
+      if constexpr (!kRest) {
+#pragma unroll
+        for (int b = 0; b < KB; ++b)
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            ur[b][e] = (b < B && lane * 8 < R) ? s_u[(b < B && lane * 8 < R) ? b * R + lane * 8 + e : 0] : 0.f;
+      }
       float* glg = p.uniforms ? p.lg + static_cast<size_t>(j & 1) * B * V : nullptr;  // sampled: final logits
       // rows read through L2 first (the longest latency): one group of rows per warp at a time.
       // kRace: a pass has kGroup x KB (row, sequence) lanes, so one perturbation per lane serves
@@ -1459,84 +1647,149 @@ __global__ void __launch_bounds__(kRollThreads, 1)
       constexpr int kBatch = 32 / kPerPass;
       float gbatch = 0.f;
       int pass = 0;
-      for (int r0 = warp * kGroup; r0 < n_g; r0 += kRollWarps * kGroup, ++pass) {
-        uint4 raw[kGroup];
+      if constexpr (kRest) {
+        // the rows past the MMA blocks: each warp's 16-row tiles, the next one's loads issued as soon as
+        // this one's fragments are consumed
+        constexpr int kSeq = RestTile<KB>::kSeq;
+        const int g = lane >> 2, t = lane & 3;
+        Lse rm[kSeq];
+        Pick rp[kSeq];
 #pragma unroll
-        for (int r = 0; r < kGroup; ++r)
-          raw[r] = (r0 + r < n_g && lane * 8 < R)
-                       ? ld16_hint(p.w2 + static_cast<size_t>(r_lo + n_t + n_s + r0 + r) * R + lane * 8, pol_rest)
-                       : make_uint4(0, 0, 0, 0);
-        float pg = 0.f;
-        if constexpr (kRace) {
-          if (pass % kBatch == 0) {
-            const int li = lane % kPerPass;
-            gbatch = lane_gumbel<KB, kRace>(p.seed, li, j,
-                                            r_lo + n_t + n_s + r0 + (lane / kPerPass) * kRollWarps * kGroup);
-          }
-          pg = __shfl_sync(0xffffffffu, gbatch, (pass % kBatch) * kPerPass + lane % kPerPass);
+        for (int i = 0; i < kSeq; ++i) {
+          rm[i] = lse_empty();
+          rp[i] = pick_empty();
         }
-        float dot[32] = {};
-        group_fma<KB, kGroup>(raw, 0, ur, dot);
-        wide_push<KB, kRace>(dot, lane, min(kGroup, n_g - r0), n_t + n_s + r0, r_lo + n_t + n_s + r0, s_base, s_b2,
-                             rows_cta, B, mine, glg, V, pmine, pg);
-      }
-      Lse st[KB];
-      Pick pst[KB];
+        for (int r0 = 16 * warp; r0 < n_g; r0 += 16 * kRollWarps) {
+          float d[2][kSeq];
+          rest.multiply(s_bop, R, lane, d);
+          if (r0 + 16 * kRollWarps < n_g)
+            rest.load(w2_rest + static_cast<size_t>(r0 + 16 * kRollWarps) * R, R, n_g - r0 - 16 * kRollWarps, lane, pol_rest);
 #pragma unroll
-      for (int b = 0; b < KB; ++b) {
-        st[b] = lse_empty();
-        pst[b] = pick_empty();
+          for (int h = 0; h < 2; ++h) {
+            const int rr = n_t + n_s + r0 + g + 8 * h;  // CTA-local row
+#pragma unroll
+            for (int i = 0; i < kSeq; ++i) {
+              const int b = t + 4 * i;
+              if (rr < r_n && b < B) {
+                const float logit = s_base[b * rows_cta + rr] + s_b2[rr] + d[h][i];
+                lse_push(rm[i], logit, r_lo + rr);
+                if constexpr (kRace)
+                  pick_push(rp[i], logit, race_gumbel(race_words(p.seed, i, j, r_lo + rr), t), r_lo + rr);
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int b = 0; b < KB; ++b) {
+          if (t == (b & 3)) {
+            lse_merge(st[b], rm[b >> 2]);
+            if constexpr (kRace) pick_merge(pst[b], rp[b >> 2]);
+          }
+        }
+      } else {
+        for (int r0 = warp * kGroup; r0 < n_g; r0 += kRollWarps * kGroup, ++pass) {
+          uint4 raw[kGroup];
+  #pragma unroll
+          for (int r = 0; r < kGroup; ++r)
+            raw[r] = (r0 + r < n_g && lane * 8 < R)
+                         ? ld16_hint(p.w2 + static_cast<size_t>(r_lo + n_t + n_s + r0 + r) * R + lane * 8, pol_rest)
+                         : make_uint4(0, 0, 0, 0);
+          float pg = 0.f;
+          if constexpr (kRace) {
+            if (pass % kBatch == 0) {
+              const int li = lane % kPerPass;
+              gbatch = lane_gumbel<KB, kRace>(p.seed, li, j,
+                                              r_lo + n_t + n_s + r0 + (lane / kPerPass) * kRollWarps * kGroup);
+            }
+            pg = __shfl_sync(0xffffffffu, gbatch, (pass % kBatch) * kPerPass + lane % kPerPass);
+          }
+          float dot[32] = {};
+          group_fma<KB, kGroup>(raw, 0, ur, dot);
+          wide_push<KB, kRace>(dot, lane, min(kGroup, n_g - r0), n_t + n_s + r0, r_lo + n_t + n_s + r0, s_base, s_b2,
+                               rows_cta, B, mine, glg, V, pmine, pg);
+        }
       }
       if constexpr (kMma) {
         // ---- epilogue: warp w reads lane quarter w % 4 of every other D block (warps w and
         //      w + 4 alternate), one row per thread, in increasing row order
-        // one row of block i: its logits from the accumulator (g0, g1: kRace, the row's
-        // perturbations for sequences 0 and 1)
-        auto epi_row = [&](int i, float g0, float g1) {
-          float d[4];
-          tc_ld_x4(tq + static_cast<uint32_t>(dcol0 + 16 * i), d);
-          tc_wait_ld();
-          const int row = 128 * i + 32 * q + lane;
-          if (row < r_n) {
+        // kRace: the perturbations of block i's row of this thread (one counter serves four sequences)
+        auto epi_gumbel = [&](int i, float (&g)[KB]) {
 #pragma unroll
-            for (int b = 0; b < KB; ++b) {
-              if (b < B) {
-                const float logit = s_base[b * rows_cta + row] + s_b2[row] + (d[2 * b] + d[2 * b + 1]);
-                if (glg) glg[static_cast<size_t>(b) * V + r_lo + row] = logit;
-                lse_push(st[b], logit, r_lo + row);
-                if constexpr (kRace) pick_push(pst[b], logit, b == 0 ? g0 : g1, r_lo + row);
-              }
+          for (int b = 0; b < KB; ++b) g[b] = 0.f;
+          if constexpr (kRace) {
+#pragma unroll
+            for (int b0 = 0; b0 < KB; b0 += 4) {
+              const uint4 x = race_words(p.seed, b0 / 4, j, r_lo + 128 * i + 32 * q + lane);
+#pragma unroll
+              for (int b = b0; b < (KB < b0 + 4 ? KB : b0 + 4); ++b) g[b] = race_gumbel(x, b - b0);
             }
           }
         };
-        // kRace: the perturbations of this thread's first kEpiRows rows, computed while the MMAs
-        // run (they depend on no data) as independent chains, without branches (a row past the
-        // CTA's blocks costs one unused chain); KB <= 2, so one counter serves the row
-        constexpr int kEpiRows = 4;
-        float gq[kEpiRows][2];
+        // A thread's rows, kEpi at a time: their logits are formed first, then one maximum and one exp a
+        // row (no chain of rescaled sums).  kRace: the first group's perturbations are computed while the
+        // MMAs run (they depend on no data) as independent chains, without branches (a row past the CTA's
+        // blocks costs one unused chain).
+        constexpr int kEpi = KB <= 4 ? 4 : 2;
+        float gq[kEpi][KB];
 #pragma unroll
-        for (int t = 0; t < kEpiRows; ++t) {
-          gq[t][0] = gq[t][1] = 0.f;
-          if constexpr (kRace) {
-            const uint4 x = race_words(p.seed, 0, j, r_lo + 128 * (half + 2 * t) + 32 * q + lane);
-            gq[t][0] = race_gumbel(x, 0);
-            gq[t][1] = KB > 1 ? race_gumbel(x, 1) : 0.f;
-          }
-        }
+        for (int t = 0; t < kEpi; ++t) epi_gumbel(half + 2 * t, gq[t]);
         const bool done = mbar_wait(&s_mma, static_cast<uint32_t>(j & 1), &s_fail, p.status);
         if (__all_sync(0xffffffffu, done)) {  // warp-uniform: the loads are .sync.aligned
           tc_fence_after();
+          for (int i0 = half; i0 < n_blk; i0 += 2 * kEpi) {
+            float x[kEpi][KB];  // logits; -inf past the CTA's rows and sequences
 #pragma unroll
-          for (int t = 0; t < kEpiRows; ++t)
-            if (half + 2 * t < n_blk) epi_row(half + 2 * t, gq[t][0], gq[t][1]);
-          for (int i = half + 2 * kEpiRows; i < n_blk; i += 2) {  // more than 8 blocks: perturbed here
-            float g0 = 0.f, g1 = 0.f;
-            if constexpr (kRace) {
-              const uint4 x = race_words(p.seed, 0, j, r_lo + 128 * i + 32 * q + lane);
-              g0 = race_gumbel(x, 0);
-              g1 = KB > 1 ? race_gumbel(x, 1) : 0.f;
+            for (int t = 0; t < kEpi; ++t) {
+              const int i = i0 + 2 * t;
+#pragma unroll
+              for (int b = 0; b < KB; ++b) x[t][b] = -INFINITY;
+              if (i < n_blk) {
+                float d[KB == 1 ? 4 : KB == 2 ? 8 : KB == 4 ? 16 : 32];
+                ld_acc<KB>(tq + static_cast<uint32_t>(dcol0 + kN * i), d);
+                tc_wait_ld();
+                const int row = 128 * i + 32 * q + lane;
+                if (row < r_n) {
+#pragma unroll
+                  for (int b = 0; b < KB; ++b) {
+                    if (b < B) {
+                      const float logit =
+                          s_base[b * rows_cta + row] + s_b2[row] + (d[3 * b] + (d[3 * b + 1] + d[3 * b + 2]));
+                      x[t][b] = logit;
+                      if constexpr (kCdf) {
+                        if (glg) glg[static_cast<size_t>(b) * V + r_lo + row] = logit;
+                        lse_push(st[b], logit, r_lo + row);
+                      }
+                    }
+                  }
+                  if constexpr (kRace) {
+                    if (i0 != half) epi_gumbel(i, gq[t]);  // further groups: perturbed here
+#pragma unroll
+                    for (int b = 0; b < KB; ++b)
+                      if (b < B) pick_push(pst[b], x[t][b], gq[t][b], r_lo + row);
+                  }
+                }
+              }
             }
-            epi_row(i, g0, g1);
+            if constexpr (!kCdf) {
+#pragma unroll
+              for (int b = 0; b < KB; ++b) {
+                float m = x[0][b];
+#pragma unroll
+                for (int t = 1; t < kEpi; ++t) m = fmaxf(m, x[t][b]);
+                if (b < B && m > -INFINITY) {
+                  Lse a;
+                  a.m = m;
+                  a.s = 0.f;
+                  a.i = 0x7fffffff;
+#pragma unroll
+                  for (int t = kEpi - 1; t >= 0; --t) {
+                    a.s += x[t][b] == m ? 1.f : __expf(x[t][b] - m);
+                    if (x[t][b] == m) a.i = r_lo + 128 * (i0 + 2 * t) + 32 * q + lane;  // the lowest of equals
+                  }
+                  lse_merge(st[b], a);
+                }
+              }
+            }
           }
         }
         tc_fence_before();  // every read of D before the next step's MMAs overwrite it
@@ -1597,17 +1850,18 @@ __global__ void __launch_bounds__(kRollThreads, 1)
           }
         }
       }
-      // the L2 rows (and, in the CUDA-core layout, every row) of this lane's sequence
-      // lane % KB; ties go to the lower id
+      if constexpr (!kRest) {
+        // the rows computed on the CUDA cores, of this lane's sequence lane % KB; ties go to the lower id
 #pragma unroll
-      for (int b = 0; b < KB; ++b) {
-        if (b == lane % KB) {
-          lse_merge(st[b], mine);
-          if constexpr (kRace) pick_merge(pst[b], pmine);
+        for (int b = 0; b < KB; ++b) {
+          if (b == lane % KB) {
+            lse_merge(st[b], mine);
+            if constexpr (kRace) pick_merge(pst[b], pmine);
+          }
         }
       }
       if (!finish_step<KB, kRace>(p, j, st, pst, s_red, s_tok, nbar, &s_fail, s_base, r_lo, r_n, rows_cta, true)) break;
-      if (j + 1 == K && (kRace || p.best)) greedy_logp<KB, kRace>(p, s_red, s_tok);
+      if (j + 1 == K && (kRace || p.best)) greedy_logp<kRace>(p, s_red, s_tok);
     }
   }
   // ---- teardown: the asynchronous copies have landed (the fill: bounded), the MMAs are done
@@ -1802,7 +2056,7 @@ __global__ void __launch_bounds__(kRollThreadsAll, 1) rollout_kernel(const Rollo
     }
     if (!finish_step<KB, kRace>(p, j, st, pst, s_red, s_tok, nbar, &s_fail, s_base, r_lo, r_n, rows_cta, false)) return;
   }
-  if (kRace || p.best) greedy_logp<KB, kRace>(p, s_red, s_tok);
+  if (kRace || p.best) greedy_logp<kRace>(p, s_red, s_tok);
 }
 
 // ================================================================ launch helpers
@@ -1823,15 +2077,21 @@ static cudaError_t launch_coop(Kern kern, const RolloutParams& p, int grid, int 
   return cudaGetLastError();
 }
 
+// The tensor-core layout's inverse-CDF instantiations, at most two sequences (rollout_cdf.cu).
+cudaError_t launch_rollout_cdf_mma(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream,
+                                   const CUtensorMap& tm);
+
 template <int KB, bool kRace>
 static cudaError_t launch_rollout_kb(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream,
                                      const CUtensorMap& tm) {
   if (use_resident(p)) {
-    if constexpr (KB <= 2) {
-      if (p.mma_tb + p.mma_sb > 0)
-        return launch_coop(rollout_resident_kernel<KB, true, kRace>, p, grid, kRollThreads, smem, stream, tm);
+    if (p.mma_tb + p.mma_sb > 0) {
+      if constexpr (!kRace) {
+        if (p.uniforms) return launch_rollout_cdf_mma(p, grid, smem, stream, tm);
+      }
+      return launch_coop(rollout_resident_kernel<KB, true, kRace, false>, p, grid, kRollThreads, smem, stream, tm);
     }
-    return launch_coop(rollout_resident_kernel<KB, false, kRace>, p, grid, kRollThreads, smem, stream, tm);
+    return launch_coop(rollout_resident_kernel<KB, false, kRace, false>, p, grid, kRollThreads, smem, stream, tm);
   }
   return launch_coop(rollout_kernel<KB, kRace>, p, grid, kRollThreadsAll, smem, stream);
 }
