@@ -18,7 +18,8 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdomino.so")
 SOURCES = ["api.cu", "tc_softmax.cu", "tc_softmax_k8.cu", "tc_store.cu", "gru.cu", "tree.cu", "verify.cu", "rollout.cu",
-           "rollout_race.cu", "rollout_cdf.cu"]
+           "rollout_race.cu", "rollout_resident_fast.cu", "rollout_resident_three.cu", "rollout_resident_race_fast.cu",
+           "rollout_resident_race_three.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -1,6 +1,7 @@
 // rollout.cu -- launch of the sequential draft loop (the kernels are in rollout_kernels.cuh): the
-// shared-memory and tensor-memory layout a launch takes, and the greedy and inverse-CDF
-// instantiations; the exponential race's are in rollout_race.cu.
+// shared-memory and tensor-memory layout a launch takes, and the streamed kernel's greedy and
+// inverse-CDF instantiations; the exponential race's are in rollout_race.cu and the resident
+// kernel's in rollout_resident_*.cu.
 #include "rollout_kernels.cuh"
 
 namespace dm {

@@ -1,6 +1,6 @@
 // rollout_kernels.cuh -- the kernels of the sequential draft loop and the launch helpers that
-// instantiate them; included by rollout.cu (greedy and inverse-CDF sampling) and rollout_race.cu
-// (the seeded exponential race), so that the two sets of instantiations compile in parallel.
+// instantiate them; included by rollout.cu, rollout_race.cu and rollout_resident_*.cu, each with its
+// own set of instantiations, so that they compile in parallel.
 // The sequential draft loop, greedy or sampled (section 4.1.2 and Fig. 3: at inference each
 // draft token is chosen from the final logits L_j = L_base_j + W2 u_j + b2 and becomes the
 // causal encoder's next input).  The base logits W_lm hidden_j of every position come first from
@@ -427,65 +427,94 @@ static __device__ bool wait_count(const unsigned* ctr, unsigned target, int* sta
 // ---- phase A: h_j = GRU(emb[t_j], h_{j-1}) (torch.nn.GRU: gates r|z|n, r multiplies
 //      W_hn h + b_hn), one warp per hidden unit q, every sequence.  With an input-projection
 //      table the three input-gate sums W_i{r,z,n} emb[t_j] are entries of row t_j of it.
+//      Bound by L2 (every CTA's units' rows of W_ih and W_hh each step, 207 KB a CTA at H = 4096),
+//      so up to four sequences share one read of a unit's rows: 22.8 -> 14.0 us a step with its barrier at B = 4,
+//      H = 4096, where each sequence had read them anew.  A sum's order is that of one sequence alone.
+template <int KB>
 __device__ __forceinline__ void gru_phase(const RolloutParams& p, const int* s_tok, const float* hprev, float* hcur,
                                           int gw, int nwarps, int lane, uint64_t pol) {
+  constexpr int kS = KB < 4 ? KB : 4;  // sequences per read of the rows
   const int B = p.B, H = p.H, Ds = p.Ds;
   for (int q = gw; q < Ds; q += nwarps) {
-    for (int b = 0; b < B; ++b) {
-      const __nv_bfloat16* x = p.emb + static_cast<size_t>(s_tok[b]) * H;
-      float ar = 0.f, az = 0.f, an = 0.f, hr = 0.f, hz = 0.f, hn = 0.f;
+    for (int b0 = 0; b0 < B; b0 += kS) {
+      // entry 8 s + v: input sums (v = 0, 1, 2 for r, z, n) and recurrent sums (v = 3, 4, 5) of
+      // sequence b0 + s
+      float acc[8 * kS];
+#pragma unroll
+      for (int i = 0; i < 8 * kS; ++i) acc[i] = 0.f;
       if (p.x_table) {
         if (lane == 0) {  // summed over the warp below with the other lanes' zeros
-          const float* xt = p.x_table + static_cast<size_t>(s_tok[b]) * 3 * Ds;
-          ar = __ldg(xt + q);
-          az = __ldg(xt + Ds + q);
-          an = __ldg(xt + 2 * Ds + q);
+#pragma unroll
+          for (int s = 0; s < kS; ++s) {
+            if (b0 + s < B) {
+              const float* xt = p.x_table + static_cast<size_t>(s_tok[b0 + s]) * 3 * Ds;
+              acc[8 * s] = __ldg(xt + q);
+              acc[8 * s + 1] = __ldg(xt + Ds + q);
+              acc[8 * s + 2] = __ldg(xt + 2 * Ds + q);
+            }
+          }
         }
       } else {
+        const __nv_bfloat16* x[kS];
+#pragma unroll
+        for (int s = 0; s < kS; ++s) x[s] = p.emb + static_cast<size_t>(s_tok[b0 + s < B ? b0 + s : b0]) * H;
 #pragma unroll 4
         for (int c = lane * 8; c < H; c += 256) {
-          float xv[8], wr[8], wz[8], wn[8];
-          bf8(x + c, xv);
+          float wr[8], wz[8], wn[8];
           bf8_hint(p.w_ih + static_cast<size_t>(q) * H + c, wr, pol);
           bf8_hint(p.w_ih + static_cast<size_t>(Ds + q) * H + c, wz, pol);
           bf8_hint(p.w_ih + static_cast<size_t>(2 * Ds + q) * H + c, wn, pol);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            ar += wr[e] * xv[e];
-            az += wz[e] * xv[e];
-            an += wn[e] * xv[e];
+          for (int s = 0; s < kS; ++s) {
+            float xv[8];
+            bf8(x[s] + c, xv);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              acc[8 * s] += wr[e] * xv[e];
+              acc[8 * s + 1] += wz[e] * xv[e];
+              acc[8 * s + 2] += wn[e] * xv[e];
+            }
           }
         }
       }
-      const float* hp = hprev + static_cast<size_t>(b) * Ds;
+      const float* hp = hprev + static_cast<size_t>(b0) * Ds;
 #pragma unroll 4
       for (int c = lane * 8; c < Ds; c += 256) {
         float wr[8], wz[8], wn[8];
         bf8_hint(p.w_hh + static_cast<size_t>(q) * Ds + c, wr, pol);
         bf8_hint(p.w_hh + static_cast<size_t>(Ds + q) * Ds + c, wz, pol);
         bf8_hint(p.w_hh + static_cast<size_t>(2 * Ds + q) * Ds + c, wn, pol);
-        // written by other CTAs in this launch: read through L2, never a stale L1 line
-        const float4 h0 = __ldcg(reinterpret_cast<const float4*>(hp + c));
-        const float4 h1 = __ldcg(reinterpret_cast<const float4*>(hp + c + 4));
-        const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          hr += wr[e] * hv[e];
-          hz += wz[e] * hv[e];
-          hn += wn[e] * hv[e];
+        for (int s = 0; s < kS; ++s) {
+          // written by other CTAs in this launch: read through L2, never a stale L1 line
+          const float* hs = hp + static_cast<size_t>(b0 + s < B ? s : 0) * Ds + c;
+          const float4 h0 = __ldcg(reinterpret_cast<const float4*>(hs));
+          const float4 h1 = __ldcg(reinterpret_cast<const float4*>(hs + 4));
+          const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            acc[8 * s + 3] += wr[e] * hv[e];
+            acc[8 * s + 4] += wz[e] * hv[e];
+            acc[8 * s + 5] += wn[e] * hv[e];
+          }
         }
       }
-      ar = warp_sum(ar); az = warp_sum(az); an = warp_sum(an);
-      hr = warp_sum(hr); hz = warp_sum(hz); hn = warp_sum(hn);
-      if (lane == 0) {
+      // one reduce-scatter (the pairwise sums of a butterfly per value), then lane s gathers its
+      // sequence's six sums
+      const float a = ReduceScatter<8 * kS, 16>::run(acc);
+      float v[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) v[i] = __shfl_sync(0xffffffffu, a, ((8 * (lane % kS) + i) * 4 / kS) & 31);
+      if (lane < kS && b0 + lane < B) {
+        const int b = b0 + lane;
         const float bir = p.b_ih ? bf2f(p.b_ih[q]) : 0.f, biz = p.b_ih ? bf2f(p.b_ih[Ds + q]) : 0.f;
         const float bin = p.b_ih ? bf2f(p.b_ih[2 * Ds + q]) : 0.f;
         const float bhr = p.b_hh ? bf2f(p.b_hh[q]) : 0.f, bhz = p.b_hh ? bf2f(p.b_hh[Ds + q]) : 0.f;
         const float bhn = p.b_hh ? bf2f(p.b_hh[2 * Ds + q]) : 0.f;
-        const float r = 1.f / (1.f + expf(-(ar + bir + hr + bhr)));
-        const float z = 1.f / (1.f + expf(-(az + biz + hz + bhz)));
-        const float n = tanhf(an + bin + r * (hn + bhn));
-        hcur[static_cast<size_t>(b) * Ds + q] = (1.f - z) * n + z * __ldcg(hp + q);
+        const float r = 1.f / (1.f + expf(-(v[0] + bir + v[3] + bhr)));
+        const float z = 1.f / (1.f + expf(-(v[1] + biz + v[4] + bhz)));
+        const float n = tanhf(v[2] + bin + r * (v[5] + bhn));
+        hcur[static_cast<size_t>(b) * Ds + q] = (1.f - z) * n + z * __ldcg(hprev + static_cast<size_t>(b) * Ds + q);
       }
     }
   }
@@ -499,6 +528,31 @@ __device__ __forceinline__ void bf4(const __nv_bfloat16* p, float (&f)[4]) {
   f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y;
 }
 
+// ---- gate functions without a branch, for phases that evaluate many of them in one thread (the
+//      library's division and tanhf branch on rare operands, which keeps the units' chains from
+//      overlapping).  As accurate as those: a reciprocal refined by one Newton step, and tanh from
+//      its Taylor series below 1/2 (through x^15, the rest under 1e-8) and from exp above.
+//      NaN and infinities come out as the library's do, except that sigmoid falls no further
+//      than e^-80.
+__device__ __forceinline__ float recip_nb(float d) {  // 1 / d, 1 <= d <= 1e35 or NaN
+  const float r = __fdividef(1.f, d);
+  return fmaf(r, fmaf(-d, r, 1.f), r);
+}
+__device__ __forceinline__ float sigmoid_nb(float x) { return recip_nb(1.f + expf(-x > 80.f ? 80.f : -x)); }
+__device__ __forceinline__ float tanh_nb(float x) {
+  const float a = fabsf(x), s = x * x;
+  float t = -929569.f / 638512875.f;
+  t = fmaf(t, s, 21844.f / 6081075.f);
+  t = fmaf(t, s, -1382.f / 155925.f);
+  t = fmaf(t, s, 62.f / 2835.f);
+  t = fmaf(t, s, -17.f / 315.f);
+  t = fmaf(t, s, 2.f / 15.f);
+  t = fmaf(t, s, -1.f / 3.f);
+  const float small = fmaf(x * s, t, x);
+  const float big = copysignf(fmaf(-2.f, recip_nb(1.f + expf(a > 40.f ? 80.f : 2.f * a)), 1.f), x);
+  return a < 0.5f ? small : big;
+}
+
 // Where unit c of a sequence's h_j lies in the CTA's shared memory: within each run of 256 units the
 // lower halves (4 units) of the lanes' 8-unit groups come first, then the upper halves, so that a
 // warp's two 16-byte reads of its groups (ub_rows) touch every bank once each.
@@ -509,60 +563,66 @@ __device__ __forceinline__ int h_slot(int c) { return (c & ~255) | ((c & 4) << 5
 //      input-gate sums are row t_j of the table, the recurrent sums W_hh h_{j-1} were computed in
 //      the previous step's phase B (gh; none at j = 0), and h_{j-1} is the CTA's own copy in
 //      shared memory, updated in place (unit q of h_j needs unit q of h_{j-1} only); four consecutive
-//      units per thread and sequence.  Bound by the latency of those loads through L2, so a thread
-//      issues the loads of up to four sequences before any arithmetic (one round trip instead of
-//      one a sequence: 5.3 -> 2.7 us a step at B = 4, H = 4096).
-template <int KB>
+//      units per thread and sequence.  Bound by those loads (24 KB a sequence through L2 into every
+//      CTA, the table's row from HBM), so an item's loads are issued before the previous item's
+//      arithmetic; the loop stays rolled (unrolled over the sequences, its straight-line code and
+//      its registers cost more than they hid).  kExact: the library's functions (the inverse-CDF rule,
+//      whose draws the last bit decides); otherwise the branch-free ones.  H = 4096, a step: 1.3 ->
+//      1.0 us at B = 1, 5.2 -> 3.5 at B = 4, 10.8 -> 7.0 at B = 8.
+struct GateIn {
+  float4 x[3], hh[3];
+};
+
+template <int KB, bool kExact>
 __device__ __forceinline__ void gates_all(const RolloutParams& p, int j, const int* s_tok, float* s_h, int hs) {
-  constexpr int kU = KB < 4 ? KB : 4;  // (sequence, unit quad) items whose loads are in flight together
-  const int B = p.B, Ds = p.Ds, D4 = Ds / 4;
+  const int B = p.B, Ds = p.Ds, D4 = Ds / 4, n = B * D4;
   const float* gh = p.gh + static_cast<size_t>((j + 1) & 1) * B * 3 * Ds;  // W_hh h_{j-1}
-  for (int e0 = threadIdx.x; e0 < B * D4; e0 += kU * kRollThreads) {
-    float4 x[kU][3], hh[kU][3];
+  auto load = [&](int e, GateIn& v) {
+    const int b = e / D4, q = (e - b * D4) * 4;
+    const float* xt = p.x_table + static_cast<size_t>(s_tok[b]) * 3 * Ds;
 #pragma unroll
-    for (int i = 0; i < kU; ++i) {
-      const int e = e0 + i * kRollThreads;
-      if (e < B * D4) {
-        const int b = e / D4, q = (e - b * D4) * 4;
-        const float* xt = p.x_table + static_cast<size_t>(s_tok[b]) * 3 * Ds;
-#pragma unroll
-        for (int g = 0; g < 3; ++g) {
-          x[i][g] = __ldg(reinterpret_cast<const float4*>(xt + g * Ds + q));
-          // written by other CTAs in this launch: read through L2
-          hh[i][g] = j > 0 ? __ldcg(reinterpret_cast<const float4*>(gh + static_cast<size_t>(b) * 3 * Ds + g * Ds + q))
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      }
+    for (int g = 0; g < 3; ++g) {
+      v.x[g] = __ldg(reinterpret_cast<const float4*>(xt + g * Ds + q));
+      // written by other CTAs in this launch: read through L2
+      v.hh[g] = j > 0 ? __ldcg(reinterpret_cast<const float4*>(gh + static_cast<size_t>(b) * 3 * Ds + g * Ds + q))
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+  };
+  constexpr bool kAhead = KB > 1;  // one sequence is one item a thread at d_s <= 1024
+  GateIn cur, next;
+  int e = threadIdx.x;
+  if (kAhead && e < n) load(e, cur);
+#pragma unroll 1
+  for (; e < n; e += kRollThreads) {
+    if (!kAhead) load(e, cur);
+    else if (e + kRollThreads < n) load(e + kRollThreads, next);
+    const int b = e / D4, q = (e - b * D4) * 4;
+    float bi[3][4], bh[3][4];
 #pragma unroll
-    for (int i = 0; i < kU; ++i) {
-      const int e = e0 + i * kRollThreads;
-      if (e < B * D4) {
-        const int b = e / D4, q = (e - b * D4) * 4;
-        float bi[3][4], bh[3][4];
-#pragma unroll
-        for (int g = 0; g < 3; ++g) {
-          if (p.b_ih) bf4(p.b_ih + g * Ds + q, bi[g]); else bi[g][0] = bi[g][1] = bi[g][2] = bi[g][3] = 0.f;
-          if (p.b_hh) bf4(p.b_hh + g * Ds + q, bh[g]); else bh[g][0] = bh[g][1] = bh[g][2] = bh[g][3] = 0.f;
-        }
-        float* hrow = s_h + static_cast<size_t>(b) * hs + h_slot(q);
-        const float4 hp = j > 0 ? *reinterpret_cast<const float4*>(hrow) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float xa[3][4] = {{x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w}, {x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w},
-                                {x[i][2].x, x[i][2].y, x[i][2].z, x[i][2].w}};
-        const float ha[3][4] = {{hh[i][0].x, hh[i][0].y, hh[i][0].z, hh[i][0].w}, {hh[i][1].x, hh[i][1].y, hh[i][1].z, hh[i][1].w},
-                                {hh[i][2].x, hh[i][2].y, hh[i][2].z, hh[i][2].w}};
-        const float hpa[4] = {hp.x, hp.y, hp.z, hp.w};
-        float out[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const float r = 1.f / (1.f + expf(-(xa[0][v] + bi[0][v] + ha[0][v] + bh[0][v])));
-          const float z = 1.f / (1.f + expf(-(xa[1][v] + bi[1][v] + ha[1][v] + bh[1][v])));
-          const float n = tanhf(xa[2][v] + bi[2][v] + r * (ha[2][v] + bh[2][v]));
-          out[v] = (1.f - z) * n + z * hpa[v];
-        }
-        *reinterpret_cast<float4*>(hrow) = make_float4(out[0], out[1], out[2], out[3]);
-      }
+    for (int g = 0; g < 3; ++g) {
+      if (p.b_ih) bf4(p.b_ih + g * Ds + q, bi[g]); else bi[g][0] = bi[g][1] = bi[g][2] = bi[g][3] = 0.f;
+      if (p.b_hh) bf4(p.b_hh + g * Ds + q, bh[g]); else bh[g][0] = bh[g][1] = bh[g][2] = bh[g][3] = 0.f;
     }
+    float* hrow = s_h + static_cast<size_t>(b) * hs + h_slot(q);
+    const float4 hp = j > 0 ? *reinterpret_cast<const float4*>(hrow) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float xa[3][4] = {{cur.x[0].x, cur.x[0].y, cur.x[0].z, cur.x[0].w}, {cur.x[1].x, cur.x[1].y, cur.x[1].z, cur.x[1].w},
+                            {cur.x[2].x, cur.x[2].y, cur.x[2].z, cur.x[2].w}};
+    const float ha[3][4] = {{cur.hh[0].x, cur.hh[0].y, cur.hh[0].z, cur.hh[0].w},
+                            {cur.hh[1].x, cur.hh[1].y, cur.hh[1].z, cur.hh[1].w},
+                            {cur.hh[2].x, cur.hh[2].y, cur.hh[2].z, cur.hh[2].w}};
+    const float hpa[4] = {hp.x, hp.y, hp.z, hp.w};
+    float out[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const float ar = xa[0][v] + bi[0][v] + ha[0][v] + bh[0][v], az = xa[1][v] + bi[1][v] + ha[1][v] + bh[1][v];
+      const float r = kExact ? 1.f / (1.f + expf(-ar)) : sigmoid_nb(ar);
+      const float z = kExact ? 1.f / (1.f + expf(-az)) : sigmoid_nb(az);
+      const float an = xa[2][v] + bi[2][v] + r * (ha[2][v] + bh[2][v]);
+      const float nn = kExact ? tanhf(an) : tanh_nb(an);
+      out[v] = (1.f - z) * nn + z * hpa[v];
+    }
+    *reinterpret_cast<float4*>(hrow) = make_float4(out[0], out[1], out[2], out[3]);
+    if (kAhead) cur = next;
   }
 }
 
@@ -736,46 +796,47 @@ static __device__ void uh_prologue(const RolloutParams& p, int gw, int nwarps, i
   }
 }
 
-// ---- phase B: u_j = SiLU(W1 [hidden_j ; h_j] + b1), one warp per rank row q, every sequence.
+// ---- phase B: u_j = SiLU(W1 [hidden_j ; h_j] + b1), one warp per (rank row q, sequence): the
+//      grid has far more warps than u has rows (6.0 -> 3.9 us a step with its barrier at B = 4,
+//      r = 256, where a warp had taken a row's sequences one after another).
 //      With uh computed before the steps the warp adds uh[b K + j][q] instead of the 4096-long
 //      hidden half of the dot.
 __device__ __forceinline__ void u_phase(const RolloutParams& p, int j, const float* hcur, int gw, int nwarps,
                                         int lane, uint64_t pol) {
   const int B = p.B, K = p.K, H = p.H, Ds = p.Ds, R = p.R;
-  for (int q = gw; q < R; q += nwarps) {
+  for (int pi = gw; pi < R * B; pi += nwarps) {
+    const int q = pi % R, b = pi / R;
     const __nv_bfloat16* w = p.w1 + static_cast<size_t>(q) * (H + Ds);
-    for (int b = 0; b < B; ++b) {
-      const __nv_bfloat16* hid = p.hidden + (static_cast<size_t>(b) * K + j) * H;
-      const float* hc = hcur + static_cast<size_t>(b) * Ds;
-      float acc = 0.f;
-      if (p.uh) {
-        // written before the steps by other CTAs of this launch (ordered by the grid barriers)
-        if (lane == 0) acc = __ldcg(p.uh + (static_cast<size_t>(b) * K + j) * R + q);
-      } else {
+    const __nv_bfloat16* hid = p.hidden + (static_cast<size_t>(b) * K + j) * H;
+    const float* hc = hcur + static_cast<size_t>(b) * Ds;
+    float acc = 0.f;
+    if (p.uh) {
+      // written before the steps by other CTAs of this launch (ordered by the grid barriers)
+      if (lane == 0) acc = __ldcg(p.uh + (static_cast<size_t>(b) * K + j) * R + q);
+    } else {
 #pragma unroll 4
-        for (int c = lane * 8; c < H; c += 256) {
-          float wv[8], xv[8];
-          bf8_hint(w + c, wv, pol);
-          bf8(hid + c, xv);
+      for (int c = lane * 8; c < H; c += 256) {
+        float wv[8], xv[8];
+        bf8_hint(w + c, wv, pol);
+        bf8(hid + c, xv);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc += wv[e] * xv[e];
-        }
+        for (int e = 0; e < 8; ++e) acc += wv[e] * xv[e];
       }
+    }
 #pragma unroll 4
-      for (int c = lane * 8; c < Ds; c += 256) {
-        float wv[8];
-        bf8_hint(w + H + c, wv, pol);
-        const float4 h0 = __ldcg(reinterpret_cast<const float4*>(hc + c));
-        const float4 h1 = __ldcg(reinterpret_cast<const float4*>(hc + c + 4));
-        const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+    for (int c = lane * 8; c < Ds; c += 256) {
+      float wv[8];
+      bf8_hint(w + H + c, wv, pol);
+      const float4 h0 = __ldcg(reinterpret_cast<const float4*>(hc + c));
+      const float4 h1 = __ldcg(reinterpret_cast<const float4*>(hc + c + 4));
+      const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc += wv[e] * hv[e];
-      }
-      acc = warp_sum(acc);
-      if (lane == 0) {
-        const float a = acc + (p.b1 ? bf2f(p.b1[q]) : 0.f);
-        p.u[static_cast<size_t>(b) * R + q] = a / (1.f + expf(-a));
-      }
+      for (int e = 0; e < 8; ++e) acc += wv[e] * hv[e];
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) {
+      const float a = acc + (p.b1 ? bf2f(p.b1[q]) : 0.f);
+      p.u[static_cast<size_t>(b) * R + q] = a / (1.f + expf(-a));
     }
   }
 }
@@ -1301,9 +1362,10 @@ __device__ __forceinline__ void ld_acc(uint32_t taddr, float (&d)[KB == 1 ? 4 : 
 // read through L2 straight into A fragments.  In each 64-column chunk lane 4 g + t loads columns
 // 16 t .. 16 t + 15 of rows g and g + 8 (32 contiguous bytes a row) and MMA step s of the chunk takes
 // words 2 s and 2 s + 1 of those; B's column g is read the same way from the swizzled B operand, so
-// both sides meet at the same columns.  Bound by L2 (512 bytes a row at about 29 B a clock and SM):
-// the first tile's loads are issued before the wait for u_j, whose latency they share.  The CUDA-core
-// form took 3.6 us a step for 232 rows at B = 1 and 8.4 us for 360 rows at B = 4.
+// both sides meet at the same columns.  Bound by L2 (512 bytes a row at about 29 B a clock and SM), so
+// a warp's first tile stays in its registers where they allow it (kHold) and the loads of the next
+// are issued before the wait for u_j, whose latency they share.  The CUDA-core form took 3.6 us a step for 232
+// rows at B = 1 and 8.4 us for 360 rows at B = 4; every tile read each step 2.7 and 3.6 us.
 template <int KB>
 struct RestTile {
   static constexpr int kNt = KB <= 2 ? 1 : KB == 4 ? 2 : 3;  // 8-column B tiles
@@ -1381,14 +1443,19 @@ struct RestTile {
 
 // kCdf (kMma only): the inverse-CDF rule, whose rows past the MMA blocks stay on the CUDA cores and
 // whose sums keep their order, since they decide the draws.
-template <int KB, bool kMma, bool kRace, bool kCdf>
+// kFast: the two-barrier step (p.fast_gates); otherwise the three-phase one.  Separate kernels, since
+// each needs the whole register budget.
+template <int KB, bool kMma, bool kRace, bool kCdf, bool kFast>
 __global__ void __launch_bounds__(kRollThreads, 1)
     rollout_resident_kernel(const RolloutParams p, const __grid_constant__ CUtensorMap tm_w2) {
   constexpr int kN = mma_n(KB);            // columns of D, rows of the B operand
   constexpr int kBopTileBytes = kN * 128;  // B operand: kN rows x 64 bf16 columns
   static_assert(3 * KB < kN, "the B operand holds three rows per sequence and a zero row");
-  static_assert(!kCdf || (kMma && !kRace && KB <= 2), "the inverse-CDF form of the tensor-core layout");
+  static_assert(!kCdf || (kMma && kFast && !kRace && KB <= 2), "the inverse-CDF form of the tensor-core layout");
   constexpr bool kRest = kMma && !kCdf;  // rows past the MMA blocks on mma.sync
+  // a tile held in registers: 64 of them, which the gates of two and more sequences need themselves
+  // (B = 4 with the table, held: 450 bytes of spills a thread and 508 -> 586 us a block)
+  constexpr bool kHold = !kFast || KB == 1;
   const int hs = (p.Ds + 255) & ~255;    // stride of a sequence's h in shared memory (h_slot)
   const int B = p.B, K = p.K, V = p.V, R = p.R;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1531,6 +1598,14 @@ __global__ void __launch_bounds__(kRollThreads, 1)
                    // the A blocks after the step's first barrier
     for (int r = tid; r < r_n; r += kRollThreads) s_b2[r] = p.b2 ? bf2f(p.b2[r_lo + r]) : 0.f;
 
+    // kHold: this warp's first tile of the rows past the MMA blocks stays in its registers for the
+    // whole block; its other tiles are read every step
+    [[maybe_unused]] const __nv_bfloat16* w2_rest = p.w2 + static_cast<size_t>(r_lo + n_t + n_s) * R;
+    [[maybe_unused]] RestTile<KB> held, rest;
+    if constexpr (kRest && kHold) held.load(w2_rest + static_cast<size_t>(16 * warp) * R, R, n_g - 16 * warp, lane, pol_once);
+    auto rest_load = [&](int r0) {
+      if (r0 < n_g) rest.load(w2_rest + static_cast<size_t>(r0) * R, R, n_g - r0, lane, l2_policy_evict_last());
+    };
     constexpr int kRows = WidePass<KB>::kRows, kGroup = WidePass<KB>::kGroup;
     const uint64_t pol_ab = l2_policy_evict_normal();
     const uint64_t pol_rest = l2_policy_evict_last();
@@ -1540,23 +1615,21 @@ __global__ void __launch_bounds__(kRollThreads, 1)
       float* hcur = p.h + static_cast<size_t>(j & 1) * B * p.Ds;
       // this step's base logits for the CTA's rows: asynchronous copies that land during A and B
       // (greedy two-barrier step: issued by the previous step's finish, from step 1 on)
-      if (j == 0 || p.best == nullptr || !p.fast_gates) {
+      if (j == 0 || p.best == nullptr || !kFast) {
         copy_base(p, j, s_base, r_lo, r_n, rows_cta);
       }
-      [[maybe_unused]] RestTile<KB> rest;  // kRest: this warp's tile of the rows past the MMA blocks
-      [[maybe_unused]] const __nv_bfloat16* w2_rest = p.w2 + static_cast<size_t>(r_lo + n_t + n_s) * R;
-      if (p.fast_gates) {
-        gates_all<KB>(p, j, s_tok, s_h, hs);
+      if constexpr (kFast) {
+        gates_all<KB, !kRest>(p, j, s_tok, s_h, hs);
         compute_sync();  // h_j of every sequence in this CTA's shared memory
         ub_phase<KB>(p, j, s_h, hs, gw, nwarps, lane, pol_ab);
-        if constexpr (kRest) rest.load(w2_rest + static_cast<size_t>(16 * warp) * R, R, n_g - 16 * warp, lane, pol_rest);
+        if constexpr (kRest) rest_load(16 * (kHold ? warp + kRollWarps : warp));
         // phase C needs u_j only: every one of its R rows counted, not a grid barrier
         if (!wait_count(p.ucount, static_cast<unsigned>(R) * (j + 1), p.status, &s_fail)) break;
       } else {
-        gru_phase(p, s_tok, hprev, hcur, gw, nwarps, lane, pol_ab);
+        gru_phase<KB>(p, s_tok, hprev, hcur, gw, nwarps, lane, pol_ab);
         if (!grid_barrier(p.barrier, nbar++, p.status, &s_fail)) break;
         u_phase(p, j, hcur, gw, nwarps, lane, pol_ab);
-        if constexpr (kRest) rest.load(w2_rest + static_cast<size_t>(16 * warp) * R, R, n_g - 16 * warp, lane, pol_rest);
+        if constexpr (kRest) rest_load(16 * (kHold ? warp + kRollWarps : warp));
         if (!grid_barrier(p.barrier, nbar++, p.status, &s_fail)) break;
       }
       if constexpr (kMma) {  // u_j as the B operand: rows 3b .. 3b + 2, four columns at a time (r % 64 == 0)
@@ -1659,11 +1732,7 @@ __global__ void __launch_bounds__(kRollThreads, 1)
           rm[i] = lse_empty();
           rp[i] = pick_empty();
         }
-        for (int r0 = 16 * warp; r0 < n_g; r0 += 16 * kRollWarps) {
-          float d[2][kSeq];
-          rest.multiply(s_bop, R, lane, d);
-          if (r0 + 16 * kRollWarps < n_g)
-            rest.load(w2_rest + static_cast<size_t>(r0 + 16 * kRollWarps) * R, R, n_g - r0 - 16 * kRollWarps, lane, pol_rest);
+        auto rest_push = [&](int r0, const float (&d)[2][kSeq]) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const int rr = n_t + n_s + r0 + g + 8 * h;  // CTA-local row
@@ -1678,6 +1747,19 @@ __global__ void __launch_bounds__(kRollThreads, 1)
               }
             }
           }
+        };
+        if constexpr (kHold) {
+          if (16 * warp < n_g) {
+            float d[2][kSeq];
+            held.multiply(s_bop, R, lane, d);
+            rest_push(16 * warp, d);
+          }
+        }
+        for (int r0 = 16 * (kHold ? warp + kRollWarps : warp); r0 < n_g; r0 += 16 * kRollWarps) {
+          float d[2][kSeq];
+          rest.multiply(s_bop, R, lane, d);
+          rest_load(r0 + 16 * kRollWarps);
+          rest_push(r0, d);
         }
 #pragma unroll
         for (int b = 0; b < KB; ++b) {
@@ -1966,7 +2048,7 @@ __global__ void __launch_bounds__(kRollThreadsAll, 1) rollout_kernel(const Rollo
     const float* hprev = p.h + static_cast<size_t>((j + 1) & 1) * B * p.Ds;  // h_{j-1} (zeros at j = 0)
     float* hcur = p.h + static_cast<size_t>(j & 1) * B * p.Ds;
     if (p.head) {
-      gru_phase(p, s_tok, hprev, hcur, gw, nwarps, lane, pol_ab);
+      gru_phase<KB>(p, s_tok, hprev, hcur, gw, nwarps, lane, pol_ab);
       if (!grid_barrier(p.barrier, nbar++, p.status, &s_fail)) return;
       u_phase(p, j, hcur, gw, nwarps, lane, pol_ab);
       if (!grid_barrier(p.barrier, nbar++, p.status, &s_fail)) return;
@@ -2077,21 +2159,45 @@ static cudaError_t launch_coop(Kern kern, const RolloutParams& p, int grid, int 
   return cudaGetLastError();
 }
 
-// The tensor-core layout's inverse-CDF instantiations, at most two sequences (rollout_cdf.cu).
-cudaError_t launch_rollout_cdf_mma(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream,
-                                   const CUtensorMap& tm);
+// The resident kernel's instantiations, each set in a unit of its own (rollout_resident_*.cu) so that
+// they compile in parallel: two-barrier and three-phase steps of the greedy (and, on the CUDA cores,
+// inverse-CDF) loop and of the race, and the inverse-CDF loop's tensor-core layout.
+#define DM_ROLL_LAUNCH(name) \
+  cudaError_t name(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream, const CUtensorMap& tm)
+DM_ROLL_LAUNCH(launch_resident_fast);
+DM_ROLL_LAUNCH(launch_resident_three);
+DM_ROLL_LAUNCH(launch_resident_race_fast);
+DM_ROLL_LAUNCH(launch_resident_race_three);
+DM_ROLL_LAUNCH(launch_rollout_cdf_mma);
+
+template <int KB, bool kRace, bool kFast>
+static cudaError_t launch_resident_kb(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream,
+                                      const CUtensorMap& tm) {
+  if (p.mma_tb + p.mma_sb > 0)
+    return launch_coop(rollout_resident_kernel<KB, true, kRace, false, kFast>, p, grid, kRollThreads, smem, stream, tm);
+  return launch_coop(rollout_resident_kernel<KB, false, kRace, false, kFast>, p, grid, kRollThreads, smem, stream, tm);
+}
+
+template <bool kRace, bool kFast>
+static cudaError_t launch_resident(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream,
+                                   const CUtensorMap& tm) {
+  if (p.B <= 1) return launch_resident_kb<1, kRace, kFast>(p, grid, smem, stream, tm);
+  if (p.B <= 2) return launch_resident_kb<2, kRace, kFast>(p, grid, smem, stream, tm);
+  if (p.B <= 4) return launch_resident_kb<4, kRace, kFast>(p, grid, smem, stream, tm);
+  return launch_resident_kb<8, kRace, kFast>(p, grid, smem, stream, tm);
+}
 
 template <int KB, bool kRace>
 static cudaError_t launch_rollout_kb(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream,
                                      const CUtensorMap& tm) {
   if (use_resident(p)) {
-    if (p.mma_tb + p.mma_sb > 0) {
-      if constexpr (!kRace) {
-        if (p.uniforms) return launch_rollout_cdf_mma(p, grid, smem, stream, tm);
-      }
-      return launch_coop(rollout_resident_kernel<KB, true, kRace, false>, p, grid, kRollThreads, smem, stream, tm);
+    if constexpr (!kRace) {
+      if (p.uniforms && p.mma_tb + p.mma_sb > 0) return launch_rollout_cdf_mma(p, grid, smem, stream, tm);
+      return p.fast_gates ? launch_resident_fast(p, grid, smem, stream, tm) : launch_resident_three(p, grid, smem, stream, tm);
+    } else {
+      return p.fast_gates ? launch_resident_race_fast(p, grid, smem, stream, tm)
+                          : launch_resident_race_three(p, grid, smem, stream, tm);
     }
-    return launch_coop(rollout_resident_kernel<KB, false, kRace, false>, p, grid, kRollThreads, smem, stream, tm);
   }
   return launch_coop(rollout_kernel<KB, kRace>, p, grid, kRollThreadsAll, smem, stream);
 }

@@ -1,5 +1,6 @@
-// rollout_race.cu -- the sequential draft loop's kernels instantiated for the seeded exponential
-// race (Gumbel-max sampling, kRace), compiled apart from rollout.cu's greedy and inverse-CDF ones.
+// rollout_race.cu -- the sequential draft loop's streamed kernel instantiated for the seeded
+// exponential race (Gumbel-max sampling, kRace), compiled apart from rollout.cu's greedy and
+// inverse-CDF ones.
 #include "rollout_kernels.cuh"
 
 namespace dm {
