@@ -21,6 +21,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <map>
@@ -203,19 +204,20 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     // The first D tiles of each CTA wait for u; the rest run whole.  Pass 0 streams only the
     // W_lm segment of those D tiles (128 x H bf16 per CTA and tile, about 6.6 TB/s over the
     // grid), so D covers the GRU's expected time (12 us + K steps of 4.5 + 0.5 B us, generous
-    // for a GRU sharing its SMs with the stream) in such tile waves, plus one.  A deferred tile
-    // never waits for the epilogue, so a larger D costs only TMEM columns ((D+2) x BN <= 512)
-    // and a later epilogue; a short estimate costs a wait at the checkpoint, never correctness.
+    // for a GRU sharing its SMs with the stream) in such tile waves, plus one.  Each deferred
+    // tile holds a TMEM block of BN columns (two spare blocks where there is room for them, so
+    // that the first whole tiles do not wait for an epilogue), so a larger D costs only TMEM
+    // columns and a later epilogue; a short estimate, or too few blocks (4 at BN = 128), costs a
+    // wait at the checkpoint, never correctness.
     {
       const double t_seg1_us = 128.0 * H * 2.0 * p.grid / 6.6e6;
       const double t_gru_us = 12.0 + K * (4.5 + 0.5 * B);
       int d = static_cast<int>(std::ceil(t_gru_us / t_seg1_us)) + 1;
-      int dmax = p.w_per_chunk < dm::kMaxDefer ? p.w_per_chunk : dm::kMaxDefer;
-      if (512 / p.bn - 2 < dmax) dmax = 512 / p.bn - 2;
+      int dmax = p.w_per_chunk < 512 / p.bn ? p.w_per_chunk : 512 / p.bn;
+      if (p.bn <= 32 && 512 / p.bn - 2 < dmax) dmax = 512 / p.bn - 2;
       p.defer_tiles = d < 1 ? 1 : (d > dmax ? dmax : d);
     }
-    p.overlap = p.u_in_gru && vsm > 0 && (p.defer_tiles + 2) * p.bn <= 512 &&
-                static_cast<size_t>(vsm) + p.gru.smem + 2048 <= 228 * 1024;
+    p.overlap = p.u_in_gru && vsm > 0 && static_cast<size_t>(vsm) + p.gru.smem + 2048 <= 228 * 1024;
     // With the overlap, chain the whole head: the gather, both projection GEMMs and the GRU
     // each let the next kernel launch early, so that the GRU's CTAs (and with them the
     // vocabulary stream) start while the projections still run.
@@ -230,7 +232,7 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
       p.fused = pairs <= dm::kGruMaxUPairs;
     }
   }
-  p.tmem_cols = pow2_at_least(p.overlap ? (p.defer_tiles + 2) * p.bn : 2 * p.bn, 32);
+  p.tmem_cols = pow2_at_least(p.overlap ? std::min((p.defer_tiles + 2) * p.bn, 512) : 2 * p.bn, 32);
 
   size_t off = 0;
   auto take = [&](size_t bytes) {

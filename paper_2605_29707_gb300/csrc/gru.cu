@@ -25,7 +25,6 @@ constexpr int kGruThreads = 256;
 constexpr int kGatePairsPerThread = 2;  // (sequence, unit) gate evaluations per thread and chunk
 constexpr int kGruWarps = kGruThreads / 32;
 constexpr int kChunkSeqs = 32;  // sequences staged per MMA pass (4 n-tiles of 8)
-constexpr int kGsmLd = kChunkSeqs + 1;  // padded row stride of the W_hh . h tile (bank spread)
 constexpr int kMaxMt = 3;  // 16-row gate tiles per CTA (up to 16 units x 3 gates)
 constexpr int kMaxNt = 4;  // 8-sequence tiles per staged chunk
 
@@ -192,29 +191,32 @@ __device__ __forceinline__ float bf_or0(const __nv_bfloat16* p, int i) {
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + expf(-x)); }
 
 // ---------------------------------------------------------------------------- smem layout
-// whh   [mt*16 rows][Ds + 8] bf16  this CTA's W_hh rows (gate g, unit jl) at row g*U + jl;
-//                                  rows past 3U are zero
+// whh   [3U (+ 1) rows][Ds + 8] bf16  this CTA's W_hh rows (gate g, unit jl) at row g*U + jl; the
+//                                  rows of the last 16-row tile past 3U share one zero row (8 units:
+//                                  25 rows instead of 32, so that the vocabulary GEMM's CTA of a
+//                                  batch of up to 128 positions fits on the same SM)
 // hsm   [chunk][Ds + 8] bf16       h_{t-1} of up to 32 sequences (the MMA's n operand)
-// gsm   [mt*16][33] f32            W_hh . h_{t-1} (padded rows)
+// gsm   [mt*16][chunk + 1] f32     W_hh . h_{t-1} (padded rows: an odd stride spreads the banks)
 // red   [8 warps][tiles][16][8] f32  k-range partial tiles of each warp
 // hprev [bc][U] f32                this CTA's own previous states (fp32)
 struct GruSmem {
   size_t whh, hsm, gsm, red, hprev, total;
-  int ldw, mt, chunk;
+  int ldw, mt, chunk, rows;
 };
 
 __host__ __device__ inline GruSmem gru_layout(int Ds, int U, int bc) {
   GruSmem L;
   L.ldw = Ds + 8;
   L.mt = (3 * U + 15) / 16;
+  L.rows = 3 * U + (L.mt * 16 > 3 * U ? 1 : 0);
   L.chunk = ((bc < kChunkSeqs ? bc : kChunkSeqs) + 7) / 8 * 8;  // staged sequences, whole n-tiles
   size_t o = 0;
   L.whh = o;
-  o += static_cast<size_t>(L.mt) * 16 * L.ldw * 2;
+  o += static_cast<size_t>(L.rows) * L.ldw * 2;
   L.hsm = o;
   o += static_cast<size_t>(L.chunk) * L.ldw * 2;
   L.gsm = o;
-  o += static_cast<size_t>(L.mt) * 16 * kGsmLd * 4;
+  o += static_cast<size_t>(L.mt) * 16 * (L.chunk + 1) * 4;
   L.red = o;  // [warp][tile][16][8] partials of each warp's k-range
   o += static_cast<size_t>(kGruWarps) * L.mt * (L.chunk / 8) * 128 * 4;
   L.hprev = o;
@@ -341,18 +343,91 @@ __device__ void fused_projections(const GruParams& p, int j0, int Uc, int b0, in
   }
 }
 
+// acc[r][i] += this lane's share of S_{m0 + r} . w[i] for NM positions (nm of them valid) and NQ rows
+// `wstride` elements apart: the tagged states are polled (other CTAs may still be publishing their
+// last step).  A lane takes 8 columns of every 256 in increasing order.  False on a timeout, the
+// same in every lane.
+template <int NM, int NQ>
+__device__ __forceinline__ bool u_dots(const GruParams& p, const __nv_bfloat16* w, int wstride, int m0, int nm,
+                                       uint32_t tag, int lane, float (&acc)[NM][NQ]) {
+  const int Ds = p.Ds;
+  bool got = true;
+  for (int c0 = 0; c0 < Ds; c0 += 4 * 256) {
+    uint4 wv[NQ][4];
+#pragma unroll
+    for (int i = 0; i < NQ; ++i)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int c = c0 + lane * 8 + k * 256;
+        if (c < Ds) wv[i][k] = __ldg(reinterpret_cast<const uint4*>(w + static_cast<size_t>(i) * wstride + c));
+      }
+#pragma unroll 1
+    for (int r = 0; r < nm; ++r) {
+      const uint32_t* srow = p.hx + static_cast<size_t>(m0 + r) * Ds;
+      uint4 sv[8];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {  // issue every load of this slice first
+        const int c = c0 + lane * 8 + k * 256;
+        if (c < Ds) {
+          sv[2 * k] = ld_relaxed_v4(srow + c);
+          sv[2 * k + 1] = ld_relaxed_v4(srow + c + 4);
+        }
+      }
+      float a[NQ];
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) {
+        a[i] = acc[0][i];
+#pragma unroll
+        for (int r2 = 1; r2 < NM; ++r2)
+          if (r2 == r) a[i] = acc[r2][i];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int c = c0 + lane * 8 + k * 256;
+        if (c >= Ds || !got) continue;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (!all_tagged(sv[2 * k + h], tag)) got = got && poll_v4(srow + c + 4 * h, sv[2 * k + h], tag);
+        const uint32_t sw[8] = {sv[2 * k].x, sv[2 * k].y, sv[2 * k].z, sv[2 * k].w,
+                                sv[2 * k + 1].x, sv[2 * k + 1].y, sv[2 * k + 1].z, sv[2 * k + 1].w};
+#pragma unroll
+        for (int i = 0; i < NQ; ++i) {
+          const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&wv[i][k]);
+#pragma unroll
+          for (int q2 = 0; q2 < 4; ++q2) {
+            const float2 wf = __bfloat1622float2(w2[q2]);
+            a[i] = fmaf(wf.x, __uint_as_float(sw[2 * q2] & 0xFFFF0000u), a[i]);
+            a[i] = fmaf(wf.y, __uint_as_float(sw[2 * q2 + 1] & 0xFFFF0000u), a[i]);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NQ; ++i)
+#pragma unroll
+        for (int r2 = 0; r2 < NM; ++r2)
+          if (r2 == r) acc[r2][i] = a[i];
+    }
+  }
+  return __all_sync(0xffffffffu, got) != 0;
+}
+
 // At most 128 registers per thread (two CTAs' worth per SM), so that a GRU CTA and a vocabulary
 // GEMM CTA (at most 168 registers x 192 threads) fit in one SM's register file.
 // kTable: the input-gate sums come from the input-projection table (p.x_table) rather than
 // from xs (a separate instantiation, so that the path without a table keeps its registers).
-// kWide: a launch that shares no SM with the vocabulary GEMM (large batches): the register
+// kX > 0 (wide): a launch that shares no SM with the vocabulary GEMM (large batches): the register
 // budget of one CTA per SM, so that a lane issues all 16 of its state loads of a step at once
 // (one L2 round trip instead of two at 16 sequences per CTA), and the steps read the input-gate
 // sums as split-K partial sums of the X GEMM directly (prefetched before each step's wait)
-// instead of a prologue pass that first sums them into xs.
-template <bool kTable, bool kWide>
-__global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const GruParams p) {
+// instead of a prologue pass that first sums them into xs.  kX of them are held per gate (further
+// ones are added at the gates): at d_s = 1024 there are at most 3 above 384 positions and 6 below,
+// where holding three, and waiting for the rest before the poll, made a step 6.8 instead of 4.7 us
+// at B = 12; holding six everywhere costs spills (B = 64: 8.7 -> 9.2 us a step).
+template <bool kTable, int kX>
+__global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const GruParams p) {
+  constexpr bool kWide = kX > 0;
   constexpr int kPollBatch = kWide ? 16 : 8;  // state loads a lane issues before checking tags
+  constexpr bool kRepoll = !kWide;
   extern __shared__ __align__(16) uint8_t gsmem[];
   const int U = p.units, Ds = p.Ds, K = p.K, B = p.B, R = p.R, H = p.H;
   const int M = B * K;
@@ -368,7 +443,7 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
   float* red = reinterpret_cast<float*>(gsmem + L.red);
   float* hprev = reinterpret_cast<float*>(gsmem + L.hprev);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ldw = L.ldw;
+  const int ldw = L.ldw, gsm_ld = L.chunk + 1;
   // This step's tag for the state words (low half): the workspace's step epoch, advanced by
   // the merge kernel at the end of every step, so that words a previous step wrote never pass
   // for this step's; 0 (a cleared word) is never a tag.
@@ -420,12 +495,12 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
     cp_async16(whh + static_cast<size_t>(g * U + jl) * ldw + c8 * 8,
                p.w_hh + (static_cast<size_t>(g) * Ds + j0 + jl) * Ds + c8 * 8);
   }
-  for (int e = tid; e < L.mt * 16 * (ldw / 8); e += kGruThreads) {
+  for (int e = tid; e < L.rows * (ldw / 8); e += kGruThreads) {
     const int r = e / (ldw / 8);
     const int jl = r % U;
     if (r >= 3 * U || jl >= Uc) reinterpret_cast<uint4*>(whh)[e] = make_uint4(0, 0, 0, 0);
   }
-  for (int r = tid; r < L.mt * 16; r += kGruThreads)  // padding columns Ds .. Ds+7 (k tail)
+  for (int r = tid; r < L.rows; r += kGruThreads)  // padding columns Ds .. Ds+7 (k tail)
     *reinterpret_cast<uint4*>(whh + static_cast<size_t>(r) * ldw + Ds) = make_uint4(0, 0, 0, 0);
   for (int e = tid; e < L.chunk * (ldw / 8); e += kGruThreads) reinterpret_cast<uint4*>(hsm)[e] = make_uint4(0, 0, 0, 0);
   __shared__ float s_uh[kGruWarps][kGruMaxUPairs];  // fused: hidden halves of this warp's u pairs
@@ -441,27 +516,32 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
   // with a table the steps read its rows; wide launches read the partial sums at each step
   const int xs_count = (kTable || kWide) ? 0 : nbc * K * 3 * Uc;
   for (int e0 = tid; e0 < xs_count; e0 += 4 * kGruThreads) {
-    float a[4];
+    float a[4], bi[4];
     size_t at[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int e = e0 + i * kGruThreads;
       a[i] = 0.f;
+      bi[i] = 0.f;
       at[i] = 0;
       if (e < xs_count) {
         const int jl = e % Uc, g = (e / Uc) % 3, bt = e / (3 * Uc);
         const int col = g * Ds + j0 + jl;
         const size_t m = static_cast<size_t>(b0) * K + bt;
         at[i] = m * 3 * Ds + col;
-        a[i] = bf_or0(p.b_ih, col);
+        bi[i] = bf_or0(p.b_ih, col);
       }
     }
+    // the partial sums in the steps' order (wide launches): 0, 3, 4, .., then 1 and 2, then b_ih
     for (int s = 0; s < p.xsplits; ++s) {
-      const float* base = p.xpart + static_cast<size_t>(s) * M * 3 * Ds;
+      const int sp = s == 0 ? 0 : s + 2 < p.xsplits ? s + 2 : s + 3 - p.xsplits;
+      const float* base = p.xpart + static_cast<size_t>(p.xsplits > 2 ? sp : s) * M * 3 * Ds;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (e0 + i * kGruThreads < xs_count) a[i] += __ldg(base + at[i]);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] += bi[i];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       if (e0 + i * kGruThreads < xs_count) p.xs[at[i]] = a[i];
@@ -493,7 +573,7 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
       const int tiles = L.mt * nt_count;
       // gate inputs of this step: issued as loads now and summed only at the gates, after the
       // wait for h_{t-1}, so that no instruction stalls on them before the wait
-      constexpr int kXr = kWide ? 3 : 1;  // X partial sums held per gate (more are summed at once)
+      constexpr int kXr = kWide ? kX : 1;
       float gx[kGatePairsPerThread][3][kXr];
 #pragma unroll
       for (int r = 0; r < kGatePairsPerThread; ++r) {
@@ -525,7 +605,6 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
 #pragma unroll
             for (int s = 0; s < kXr; ++s)
               if (s < nsplit) gx[r][g][s] = x[s * split_stride + g * Ds + j];
-            for (int s = kXr; s < nsplit; ++s) gx[r][g][0] += x[s * split_stride + g * Ds + j];  // rare
           }
         }
       }
@@ -538,6 +617,8 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
         const int q0 = kw0 * 4, q1 = min(kw1 * 4, Ds / 4);  // 4-word columns of the range
         const int ncq = max(0, q1 - q0);
         const int total = nb * ncq;
+        // (every CTA reads the states in the same order: with a starting sequence of its own each,
+        // the same lines were no longer asked for together and a step took 7.8 instead of 5.6 us at B = 32)
         bool got = true;
         for (int e0 = lane; e0 < total && got; e0 += kPollBatch * 32) {
           uint4 v[kPollBatch];
@@ -557,6 +638,18 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
               if (!all_tagged(v[i], tag)) {
                 const size_t m = static_cast<size_t>(b0 + c0 + bb) * K + (t - 1);
                 got = poll_v4(p.hx + m * Ds + cq * 4, v[i], tag);
+                // the batch was early: by now its other late words are probably there, so they are
+                // read again together rather than one round trip after another
+                if (kRepoll) {
+#pragma unroll
+                  for (int i2 = 0; i2 < kPollBatch; ++i2) {
+                    const int e2 = e0 + i2 * 32;
+                    if (i2 > i && e2 < total && !all_tagged(v[i2], tag)) {
+                      const size_t m2 = static_cast<size_t>(b0 + c0 + e2 / ncq) * K + (t - 1);
+                      v[i2] = ld_relaxed_v4(p.hx + m2 * Ds + (q0 + e2 % ncq) * 4);
+                    }
+                  }
+                }
               }
               *reinterpret_cast<uint2*>(hsm + static_cast<size_t>(bb) * ldw + cq * 4) =
                   make_uint2(pack_hi_halves(v[i].x, v[i].y), pack_hi_halves(v[i].z, v[i].w));
@@ -571,7 +664,7 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
           for (int a = 0; a < kMaxMt; ++a)
 #pragma unroll
             for (int b = 0; b < kMaxNt; ++b) acc[a][b][0] = acc[a][b][1] = acc[a][b][2] = acc[a][b][3] = 0.f;
-          const __nv_bfloat16* abase = whh + static_cast<size_t>(lane & 15) * ldw + (lane >> 4) * 8;
+          const __nv_bfloat16* abase = whh + (lane >> 4) * 8;
           const __nv_bfloat16* bbase = hsm + static_cast<size_t>(lane & 7) * ldw + ((lane >> 3) & 1) * 8;
           for (int kb = kw0; kb < kw1; ++kb) {
             uint32_t bf[kMaxNt][2];
@@ -582,7 +675,7 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
             for (int mt = 0; mt < kMaxMt; ++mt) {
               if (mt >= L.mt) break;
               uint32_t af[4];
-              ldmatrix_x4(af, abase + static_cast<size_t>(mt * 16) * ldw + kb * 16);
+              ldmatrix_x4(af, abase + static_cast<size_t>(min(mt * 16 + (lane & 15), L.rows - 1)) * ldw + kb * 16);
 #pragma unroll
               for (int nt = 0; nt < kMaxNt; ++nt)
                 if (nt < nt_count) mma_16816(acc[mt][nt], af, bf[nt]);
@@ -615,7 +708,7 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
 #pragma unroll
           for (int ww = 0; ww < kGruWarps; ++ww) sum += red[(static_cast<size_t>(ww) * tiles + tile) * 128 + w];
           const int mt = tile / nt_count, nt = tile % nt_count;
-          gsm[static_cast<size_t>(mt * 16 + w / 8) * kGsmLd + nt * 8 + (w % 8)] = sum;
+          gsm[static_cast<size_t>(mt * 16 + w / 8) * gsm_ld + nt * 8 + (w % 8)] = sum;
         }
         __syncthreads();
       }
@@ -630,16 +723,22 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
         const size_t m = static_cast<size_t>(b0 + bl) * K + t;
         float hr = bhh[rr][0], hz = bhh[rr][1], hn = bhh[rr][2];
         if (t > 0) {
-          hr += gsm[static_cast<size_t>(jl) * kGsmLd + bb];
-          hz += gsm[static_cast<size_t>(U + jl) * kGsmLd + bb];
-          hn += gsm[static_cast<size_t>(2 * U + jl) * kGsmLd + bb];
+          hr += gsm[static_cast<size_t>(jl) * gsm_ld + bb];
+          hz += gsm[static_cast<size_t>(U + jl) * gsm_ld + bb];
+          hn += gsm[static_cast<size_t>(2 * U + jl) * gsm_ld + bb];
         }
         float xin[3];
 #pragma unroll
         for (int g = 0; g < 3; ++g) {
           float s = gx[rr][g][0];
+          if constexpr (kXr > 1) {  // partial sums 0, 3, 4, ..., then 1 and 2
 #pragma unroll
-          for (int q = 1; q < kXr; ++q) s += gx[rr][g][q];
+            for (int q = 3; q < kXr; ++q) s += gx[rr][g][q];
+            if (!kTable)
+              for (int q = kXr; q < p.xsplits; ++q) s += p.xpart[(q * static_cast<size_t>(M) + m) * 3 * Ds + g * Ds + j];
+            s += gx[rr][g][1];
+            s += gx[rr][g][2];
+          }
           xin[g] = s + bih[rr][g];
         }
         const float hp = hprev[bl * U + jl];
@@ -663,61 +762,70 @@ __global__ void __launch_bounds__(kGruThreads, kWide ? 1 : 2) gru_kernel(const G
   //      tagged states (polled: other CTAs may still be publishing their last step)
   const int total_warps = gridDim.x * kGruWarps;
   const int gw = blockIdx.x * kGruWarps + warp;
-  const int groups = max(1, total_warps / R);
-  int np = 0;  // this warp's pair counter (the fused prologue's order)
-  for (int pi = gw; pi < R * groups; pi += total_warps) {
-    const int q = pi % R, mg = pi / R;
-    const __nv_bfloat16* w1row = p.w1 + static_cast<size_t>(q) * (H + Ds) + H;
-    const float bq = bf_or0(p.b1, q);
-    for (int m = mg; m < M; m += groups) {
-      const uint32_t* srow = p.hx + static_cast<size_t>(m) * Ds;
-      float acc = 0.f;
-      bool got = true;
-      for (int c0 = lane * 8; c0 < Ds && got; c0 += 4 * 256) {
-        uint4 wv[4], sv[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {  // issue every load of this slice first
-          const int c = c0 + i * 256;
-          if (c < Ds) {
-            wv[i] = __ldg(reinterpret_cast<const uint4*>(w1row + c));
-            sv[2 * i] = ld_relaxed_v4(srow + c);
-            sv[2 * i + 1] = ld_relaxed_v4(srow + c + 4);
-          }
+  if (p.ids != nullptr) {
+    // fused projections: the (q, m) pairs whose hidden halves this warp computed in the prologue
+    const int groups = max(1, total_warps / R);
+    int np = 0;  // this warp's pair counter (the prologue's order)
+    for (int pi = gw; pi < R * groups; pi += total_warps) {
+      const int q = pi % R, mg = pi / R;
+      const __nv_bfloat16* w1row = p.w1 + static_cast<size_t>(q) * (H + Ds) + H;
+      const float bq = bf_or0(p.b1, q);
+      for (int m = mg; m < M; m += groups) {
+        float acc[1][1] = {{0.f}};
+        if (!u_dots<1, 1>(p, w1row, 0, m, 1, tag, lane, acc)) {
+          if (lane == 0) set_status(p.status, kStatusTimeout);
+          return;
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int c = c0 + i * 256;
-          if (c >= Ds || !got) continue;
-          for (int h = 0; h < 2; ++h) {
-            uint4& x = sv[2 * i + h];
-            if (!all_tagged(x, tag)) got = got && poll_v4(srow + c + 4 * h, x, tag);
-          }
-          const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&wv[i]);
-          const uint32_t sw[8] = {sv[2 * i].x, sv[2 * i].y, sv[2 * i].z, sv[2 * i].w,
-                                  sv[2 * i + 1].x, sv[2 * i + 1].y, sv[2 * i + 1].z, sv[2 * i + 1].w};
-#pragma unroll
-          for (int q2 = 0; q2 < 4; ++q2) {
-            const float2 wf = __bfloat1622float2(w2[q2]);
-            acc = fmaf(wf.x, __uint_as_float(sw[2 * q2] & 0xFFFF0000u), acc);
-            acc = fmaf(wf.y, __uint_as_float(sw[2 * q2 + 1] & 0xFFFF0000u), acc);
-          }
-        }
-      }
-      if (__any_sync(0xffffffffu, !got)) {
-        if (lane == 0) set_status(p.status, kStatusTimeout);
-        return;
-      }
-      if (p.ids != nullptr) {
-        if (lane == 0 && np < kGruMaxUPairs) acc += s_uh[warp][np];
+        if (lane == 0 && np < kGruMaxUPairs) acc[0][0] += s_uh[warp][np];
         ++np;
-      } else {
-        for (int s = lane; s < p.usplits; s += 32) acc += __ldg(p.upart + (static_cast<size_t>(s) * M + m) * R + q);
+        const float sum = warp_sum(acc[0][0]);
+        if (lane == 0) {
+          const float a = sum + bq;
+          p.u[static_cast<size_t>(m) * R + q] = __float2bfloat16_rn(a / (1.f + expf(-a)));
+        }
       }
-      acc = warp_sum(acc);
-      if (lane == 0) {
-        const float a = acc + bq;
-        p.u[static_cast<size_t>(m) * R + q] = __float2bfloat16_rn(a / (1.f + expf(-a)));
+    }
+    return;
+  }
+  // 4 rank rows x 4 positions per warp: each W1 row and state row is read through L2 once for four
+  // products (a pair at a time, every warp read 6 KB and 64 scattered partial sums for each product:
+  // 24 us at B = 4, 44 us at B = 8, bound by L2)
+  const int qt = R / 4, mt4 = (M + 3) / 4;  // R is a multiple of 8
+  for (int ti = gw; ti < qt * mt4; ti += total_warps) {
+    const int q0 = 4 * (ti % qt), m0 = 4 * (ti / qt);
+    const int nm = min(4, M - m0);
+    float acc[4][4];  // [position][row]
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[r][i] = 0.f;
+    if (!u_dots<4, 4>(p, p.w1 + static_cast<size_t>(q0) * (H + Ds) + H, H + Ds, m0, nm, tag, lane, acc)) {
+      if (lane == 0) set_status(p.status, kStatusTimeout);
+      return;
+    }
+    for (int s = lane; s < p.usplits; s += 32) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (r < nm) {
+          const float4 v = __ldg(reinterpret_cast<const float4*>(p.upart + (static_cast<size_t>(s) * M + m0 + r) * R + q0));
+          acc[r][0] += v.x;
+          acc[r][1] += v.y;
+          acc[r][2] += v.z;
+          acc[r][3] += v.w;
+        }
       }
+    }
+    float mine = 0.f;  // lane 4 r + i: the sum of (position r, row i)
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float sum = warp_sum(acc[r][i]);
+        if (lane == 4 * r + i) mine = sum;
+      }
+    if (lane < 4 * nm) {
+      const float a = mine + bf_or0(p.b1, q0 + (lane & 3));
+      p.u[static_cast<size_t>(m0 + (lane >> 2)) * R + q0 + (lane & 3)] = __float2bfloat16_rn(a / (1.f + expf(-a)));
     }
   }
 }
@@ -742,11 +850,11 @@ GruPlan gru_plan(int B, int Ds, int num_sms) {
   return g;
 }
 
-template <bool kTable, bool kWide>
+template <bool kTable, int kX>
 static cudaError_t launch_gru_t(const GruParams& p, const GruPlan& plan, cudaStream_t stream, bool pdl) {
   {
     const cudaError_t e =
-        ensure_smem_attr(reinterpret_cast<const void*>(gru_kernel<kTable, kWide>), plan.smem, true);
+        ensure_smem_attr(reinterpret_cast<const void*>(gru_kernel<kTable, kX>), plan.smem, true);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
@@ -763,12 +871,12 @@ static cudaError_t launch_gru_t(const GruParams& p, const GruPlan& plan, cudaStr
   // A runtime that refuses the pair gets the cooperative launch alone from then on.
   static std::atomic<bool> pdl_refused{false};
   cfg.numAttrs = (pdl && !pdl_refused) ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kWide>, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kX>, p);
   if (e != cudaSuccess && cfg.numAttrs == 2) {
     (void)cudaGetLastError();
     pdl_refused = true;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kWide>, p);
+    e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kX>, p);
   }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -777,9 +885,10 @@ static cudaError_t launch_gru_t(const GruParams& p, const GruPlan& plan, cudaStr
 cudaError_t launch_gru(const GruParams& p, const GruPlan& plan, cudaStream_t stream, bool pdl, bool wide) {
   if (plan.smem == 0) return cudaErrorInvalidValue;
   if (wide && p.ids != nullptr) return cudaErrorInvalidValue;  // fused projections share SMs
-  if (wide)
-    return p.x_table ? launch_gru_t<true, true>(p, plan, stream, pdl) : launch_gru_t<false, true>(p, plan, stream, pdl);
-  return p.x_table ? launch_gru_t<true, false>(p, plan, stream, pdl) : launch_gru_t<false, false>(p, plan, stream, pdl);
+  if (!wide)
+    return p.x_table ? launch_gru_t<true, 0>(p, plan, stream, pdl) : launch_gru_t<false, 0>(p, plan, stream, pdl);
+  if (p.x_table) return launch_gru_t<true, 1>(p, plan, stream, pdl);
+  return p.xsplits <= 3 ? launch_gru_t<false, 3>(p, plan, stream, pdl) : launch_gru_t<false, 6>(p, plan, stream, pdl);
 }
 
 // ---------------------------------------------------------------------------- u finalize

@@ -15,9 +15,9 @@ enum TcMode { kModeSoftmax = 0, kModeStore = 1 };
 // and size; safe to call from several host threads (api.cu).
 cudaError_t ensure_smem_attr(const void* func, size_t smem, bool carveout);
 
-// Most deferred tiles one CTA of the vocabulary GEMM can hold (each has its own completion
-// barrier in shared memory).
-constexpr int kMaxDefer = 32;
+// Most accumulator blocks (of at least 16 tensor-memory columns) one CTA of a GEMM holds, and so the
+// most tiles of the vocabulary GEMM that can wait for their second segment.
+constexpr int kMaxBlocks = 32;
 
 // One tcgen05 GEMM launch: acc[tok, w] = sum over two K segments of
 //   seg1: X1[tok, :] . W1[w, :]      (k blocks 0 .. nkb1-1)
@@ -60,7 +60,7 @@ cudaError_t launch_tc_gemm(int mode, int bn, bool swap, int kmax, const CUtensor
 // of the kernel before it (p.pdl_wait says where it waits for that kernel).
 cudaError_t launch_tc_store_dependent(const CUtensorMap* maps, const TcParams& p, int grid, cudaStream_t stream);
 // Deferred-segment vocabulary GEMM launched as a programmatic dependent of the GRU kernel
-// (bn 16 or 32; fewer pipeline stages so that its CTAs fit beside the GRU's on one SM).
+// (bn 16 to 128; fewer pipeline stages so that its CTAs fit beside the GRU's on one SM).
 cudaError_t launch_tc_softmax_deferred(int bn, int kmax, const CUtensorMap* maps, const TcParams& p, int grid,
                                        cudaStream_t stream);
 // Shared memory one deferred-mode CTA uses (for the co-residency budget).

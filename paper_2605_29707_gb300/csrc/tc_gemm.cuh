@@ -3,14 +3,14 @@
 // Warp roles (192 threads):
 //   warp 0      one thread issues TMA tile loads into a STAGES-deep shared-memory ring;
 //   warp 1      allocates TMEM; one thread issues tcgen05.mma (M = 128, N = BN, K = 16 per
-//               instruction) into one of two TMEM accumulators and commits to mbarriers;
+//               instruction) into a TMEM accumulator block and commits to mbarriers;
 //   warps 2..5  epilogue: tcgen05.ld the finished accumulator and either
 //               - softmax mode: fold every logit into a per-(token, CTA) running max, running
 //                 sum of exp and a top-KMAX list (value desc, id asc), so that the logits never
 //                 leave the chip (the vocabulary projection of section 4.1.1 plus the W2 term
 //                 of section 4.1.2 in one accumulator), or
 //               - store mode: write fp32 partial sums (split-K) of a plain projection.
-// The two accumulators let the epilogue of tile i overlap the main loop of tile i+1.
+// The accumulator blocks let the epilogue of tile i overlap the main loop of tile i+1.
 #pragma once
 
 #include <math.h>
@@ -31,14 +31,18 @@ struct TcCfg {
   static constexpr int kBBytes = BN * 128;   // BN rows x 64 bf16
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kTPT = SWAP ? 128 / BN : 1;  // epilogue threads per token (swap)
-  static constexpr int kTrStride = 128 + kTPT;      // conflict-free transpose pitch (floats)
+  // Vocabulary rows transposed at a time: what gives each epilogue thread one chunk of 32 values
+  // (16 for BN = 16).  A whole 128-row tile at BN = 64 and 128 would take 33 and 66 KB of shared
+  // memory instead of 17, which the ring needs (and, in the deferred variants, the GRU's CTA).
+  static constexpr int kTrRows = 32 * kTPT < 128 ? 32 * kTPT : 128;
+  static constexpr int kTrStride = kTrRows + kTPT;  // conflict-free transpose pitch (floats)
   static constexpr int kTrBytes = (SWAP && MODE == kModeSoftmax) ? BN * kTrStride * 4 : 0;
   static constexpr int kBudget = 200 * 1024;
   static constexpr int kSt0 = (kBudget - kTrBytes) / kStageBytes;
   static constexpr int kStages = ST > 0 ? ST : (kSt0 > 8 ? 8 : kSt0);
   static constexpr int kTmemCols =
       (2 * BN <= 32) ? 32 : (2 * BN <= 64) ? 64 : (2 * BN <= 128) ? 128 : (2 * BN <= 256) ? 256 : 512;
-  static constexpr int kBarBytes = 512;  // ring, accumulator and per-deferred-tile barriers
+  static constexpr int kBarBytes = 1024;  // ring barriers and two per accumulator block
   // per-thread scratch of one 32-value chunk (rare path of the normal orientation)
   static constexpr int kListBytes = (MODE == kModeSoftmax && !SWAP) ? 128 * 32 * 4 : 0;
   static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kTrBytes + kListBytes + kBarBytes;
@@ -81,14 +85,12 @@ __device__ __forceinline__ bool tc_get_item(const TcParams& p, int i, TcItem& it
   }
 }
 
-// TMEM column of item i's accumulator: two alternating buffers; in deferred mode the first
-// p.defer tiles each keep their own column block (holding the first segment until the second
-// is added) and later tiles alternate between the two blocks after them.
+// Accumulator blocks of BN columns in the CTA's tensor memory (a power of two): item i uses block
+// i % blocks, again and again.  Two without deferral; more let the first p.defer items hold their first
+// segment until the second is added.
 template <int BN>
-__device__ __forceinline__ uint32_t tc_acc_col(const TcParams& p, int i) {
-  if (!p.defer) return static_cast<uint32_t>((i & 1) * BN);
-  if (i < p.defer) return static_cast<uint32_t>(i * BN);
-  return static_cast<uint32_t>((p.defer + ((i - p.defer) & 1)) * BN);
+__device__ __forceinline__ int tc_blocks(const TcParams& p) {
+  return p.tmem_cols / BN;
 }
 
 // Running log-sum-exp state and top-KMAX list of one token over a stream of logits.
@@ -243,10 +245,12 @@ __device__ __forceinline__ bool epi_any(bool pred) {
   return r != 0;
 }
 
-// Deferred variants (ST > 0) must fit their registers beside a GRU CTA on one SM: the bound of
-// two CTAs per SM caps them at 168 registers per thread.
+// Deferred variants (ST > 0) must fit their registers beside a GRU CTA on one SM, which takes half of
+// them: a bound of two CTAs of 256 threads caps these at 128 a thread.  (Registers are handed out to
+// warps four at a time, so the six warps count as eight: at 168 a thread, the most that a bound of
+// two 192-thread CTAs allows, the two kernels do not share an SM.)
 template <int BN, bool SWAP, int MODE, int KMAX, int ST>
-__global__ void __launch_bounds__(192, ST > 0 ? 2 : 1)
+__global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
                    const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                    const TcParams p) {
@@ -261,10 +265,9 @@ __global__ void __launch_bounds__(192, ST > 0 ? 2 : 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(scratch) + C::kListBytes);
   uint64_t* full = bars;
   uint64_t* empty = bars + C::kStages;
-  uint64_t* tfull = bars + 2 * C::kStages;
-  uint64_t* tempty = tfull + 2;
-  uint64_t* tdone = tempty + 2;  // deferred tile i < p.defer: its accumulator is complete
-  uint64_t* drain = tdone + kMaxDefer;
+  uint64_t* tfull = bars + 2 * C::kStages;  // accumulator block finished
+  uint64_t* tempty = tfull + kMaxBlocks;    // accumulator block drained by the epilogue
+  uint64_t* drain = tempty + kMaxBlocks;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -276,11 +279,10 @@ __global__ void __launch_bounds__(192, ST > 0 ? 2 : 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], p.mcast > 1 ? p.mcast : 1);  // every CTA of a multicast cluster releases it
     }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < tc_blocks<BN>(p); ++a) {
       mbar_init(&tfull[a], 1);
       mbar_init(&tempty[a], 128);
     }
-    for (int d = 0; d < kMaxDefer; ++d) mbar_init(&tdone[d], 1);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -389,16 +391,13 @@ __global__ void __launch_bounds__(192, ST > 0 ? 2 : 1)
       for (int pass = 0; pass < passes && ok; ++pass) {
       for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE>(p, i, it); ++i) {
         if (pass < 2 && p.defer && i >= p.defer) break;
-        // A deferred tile (i < p.defer) keeps its own TMEM block and signals its own barrier,
-        // so it never waits for the epilogue; later tiles take turns on two blocks.
-        const bool own = p.defer && i < p.defer;
-        const int jd = own ? 0 : i - p.defer;
-        const int ab = jd & 1;
-        const uint32_t aph = (jd >> 1) & 1;
+        // a deferred tile (i < p.defer <= blocks) is its block's first; a block used before waits
+        // for the epilogue of the tile it held
+        const int nblk = tc_blocks<BN>(p), ab = i & (nblk - 1);
         const bool last_pass = !p.defer || pass >= 1;  // passes that finish a tile
-        const uint32_t d_tmem = tmem_base + tc_acc_col<BN>(p, i);
-        if (last_pass && !own) {
-          if (!mbar_wait(&tempty[ab], aph ^ 1u, abort_flag, p.status)) break;
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ab * BN);
+        if (i >= nblk) {
+          if (!mbar_wait(&tempty[ab], (i / nblk - 1) & 1, abort_flag, p.status)) break;
           tc_fence_after();
         }
         const int kb_lo = (p.defer && pass == 1) ? p.nkb1 : it.kb0;
@@ -417,7 +416,7 @@ __global__ void __launch_bounds__(192, ST > 0 ? 2 : 1)
           else tc_commit(&empty[stage]);
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
         }
-        if (ok && last_pass) tc_commit(own ? &tdone[i] : &tfull[ab]);
+        if (ok && last_pass) tc_commit(&tfull[ab]);
       }
       }
     }
@@ -433,15 +432,11 @@ __global__ void __launch_bounds__(192, ST > 0 ? 2 : 1)
     TcItem it;
     it.tok = 0;
     for (int i = 0; tc_get_item<MODE>(p, i, it); ++i) {
-      const bool own = p.defer && i < p.defer;
-      const int jd = own ? 0 : i - p.defer;
-      const int ab = jd & 1;
-      const uint32_t aph = (jd >> 1) & 1;
-      const bool ok = own ? mbar_wait(&tdone[i], 0u, abort_flag, p.status)
-                          : mbar_wait(&tfull[ab], aph, abort_flag, p.status);
+      const int nblk = tc_blocks<BN>(p), ab = i & (nblk - 1);
+      const bool ok = mbar_wait(&tfull[ab], (i / nblk) & 1, abort_flag, p.status);
       if (epi_any(!ok)) { aborted = true; break; }
       tc_fence_after();
-      const uint32_t tcol = tmem_base + lane_off + tc_acc_col<BN>(p, i);
+      const uint32_t tcol = tmem_base + lane_off + static_cast<uint32_t>(ab * BN);
 
       if constexpr (MODE == kModeStore) {
         if constexpr (SWAP) {
@@ -483,40 +478,40 @@ __global__ void __launch_bounds__(192, ST > 0 ? 2 : 1)
         tc_fence_before();
         mbar_arrive(&tempty[ab]);
       } else if constexpr (SWAP) {
-        // vocabulary rows on TMEM lanes, tokens on columns: stage through shared memory so
-        // that each thread owns one token and a strided slice of the tile's vocabulary
+        // vocabulary rows on TMEM lanes, tokens on columns: stage kTrRows rows at a time through
+        // shared memory so that each thread owns one token and a strided slice of the rows
         const int vrow = 32 * q + lane;
         const int v = it.w * 128 + vrow;
         const bool vvalid = v < p.rows_w;
         const float bv = (p.bias != nullptr && vvalid) ? __bfloat162float(p.bias[v]) : 0.f;
-#pragma unroll
-        for (int c0 = 0; c0 < BN; c0 += (BN < 32 ? BN : 32)) {
-          float r[BN < 32 ? 16 : 32];
-          if constexpr (BN < 32) tc_ld_x16(tcol + c0, r); else tc_ld_x32(tcol + c0, r);
-          tc_wait_ld();
-#pragma unroll
-          for (int j = 0; j < (BN < 32 ? 16 : 32); ++j) tr[(c0 + j) * C::kTrStride + vrow] = r[j] + bv;
-        }
-        tc_fence_before();
-        if (!own) mbar_arrive(&tempty[ab]);  // a deferred tile's block is never reused
-        named_bar_sync(1, 128);
         const int tt = ep / C::kTPT;
         const int sub = ep % C::kTPT;
-        const int vbase = it.w * 128;
         const float* trow = tr + tt * C::kTrStride;
-        const int left = p.rows_w - vbase - sub;  // valid entries: sub + TPT * jj < rows_w - vbase
-        const int nvalid_all = left <= 0 ? 0 : (left + C::kTPT - 1) / C::kTPT;
         constexpr int kSub = BN < 32 ? BN : 32;
 #pragma unroll 1
-        for (int j0 = 0; j0 < BN; j0 += kSub) {
-          float r[kSub];
-          const float* sx = trow + sub + C::kTPT * j0;
+        for (int h0 = 0; h0 < 128; h0 += C::kTrRows) {
+          if (vrow >= h0 && vrow < h0 + C::kTrRows) {  // whole warps: kTrRows is a multiple of 32
 #pragma unroll
-          for (int j = 0; j < kSub; ++j) r[j] = sx[C::kTPT * j];
-          stream_chunk<kSub, KMAX>(r, sx, C::kTPT, vbase + sub + C::kTPT * j0, C::kTPT, nvalid_all - j0, st.mx, st.se,
-                                   st.tv, st.ti);
+            for (int c0 = 0; c0 < BN; c0 += kSub) {
+              float r[kSub];
+              if constexpr (BN < 32) tc_ld_x16(tcol + c0, r); else tc_ld_x32(tcol + c0, r);
+              tc_wait_ld();
+#pragma unroll
+              for (int j = 0; j < kSub; ++j) tr[(c0 + j) * C::kTrStride + vrow - h0] = r[j] + bv;
+            }
+            tc_fence_before();
+            mbar_arrive(&tempty[ab]);
+          }
+          named_bar_sync(1, 128);
+          const int vbase = it.w * 128 + h0 + sub;
+          const int left = p.rows_w - vbase;  // valid entries: vbase + TPT * j < rows_w
+          const int nvalid = left <= 0 ? 0 : (left + C::kTPT - 1) / C::kTPT;
+          float r[kSub];
+#pragma unroll
+          for (int j = 0; j < kSub; ++j) r[j] = trow[sub + C::kTPT * j];
+          stream_chunk<kSub, KMAX>(r, trow + sub, C::kTPT, vbase, C::kTPT, nvalid, st.mx, st.se, st.tv, st.ti);
+          named_bar_sync(1, 128);
         }
-        named_bar_sync(1, 128);
       } else {
         // tokens on TMEM lanes: each thread streams its own row across the vocabulary tile
 #pragma unroll 1

@@ -25,25 +25,27 @@ cudaError_t launch_tc_softmax(int bn, bool swap, int kmax, const CUtensorMap* ma
   return cudaErrorInvalidValue;
 }
 
-// Deferred variants: 6 stages (BN 16) / 5 stages (BN 32) keep a CTA near 118 KB of shared
-// memory so that it fits on an SM next to a GRU CTA.
+// Deferred variants: the stages that leave a GRU CTA (80 KB) room on the same SM -- 6, 5, 5 and 4 for
+// BN = 16, 32, 64 and 128 (118 to 150 KB).
 cudaError_t launch_tc_softmax_deferred(int bn, int kmax, const CUtensorMap* maps, const TcParams& p, int grid,
                                        cudaStream_t s) {
-  if (p.defer < 1 || p.defer > kMaxDefer) return cudaErrorInvalidValue;
+  if (p.defer < 1 || p.defer > kMaxBlocks || p.defer * bn > p.tmem_cols) return cudaErrorInvalidValue;
   if (kmax == 8) return launch_tc_softmax_deferred_k8(bn, maps, p, grid, s);
-  if (bn == 16 && kmax == 16) return launch_tc_instance<16, true, kModeSoftmax, 16, 6>(maps, p, grid, s, true);
-  if (bn == 16 && kmax == 32) return launch_tc_instance<16, true, kModeSoftmax, 32, 6>(maps, p, grid, s, true);
-  if (bn == 32 && kmax == 16) return launch_tc_instance<32, true, kModeSoftmax, 16, 5>(maps, p, grid, s, true);
-  if (bn == 32 && kmax == 32) return launch_tc_instance<32, true, kModeSoftmax, 32, 5>(maps, p, grid, s, true);
+#define DM_SD(BN, KM, ST) \
+  if (bn == BN && kmax == KM) return launch_tc_instance<BN, true, kModeSoftmax, KM, ST>(maps, p, grid, s, true);
+  DM_SD(16, 16, 6) DM_SD(16, 32, 6) DM_SD(32, 16, 5) DM_SD(32, 32, 5)
+  DM_SD(64, 16, 5) DM_SD(64, 32, 5) DM_SD(128, 16, 4) DM_SD(128, 32, 4)
+#undef DM_SD
   return cudaErrorInvalidValue;
 }
 
 int tc_softmax_deferred_smem(int bn, int kmax) {
   if (kmax == 8) return tc_softmax_deferred_smem_k8(bn);
-  if (bn == 16) return kmax <= 16 ? TcCfg<16, true, kModeSoftmax, 16, 6>::kSmemBytes
-                                  : TcCfg<16, true, kModeSoftmax, 32, 6>::kSmemBytes;
-  if (bn == 32) return kmax <= 16 ? TcCfg<32, true, kModeSoftmax, 16, 5>::kSmemBytes
-                                  : TcCfg<32, true, kModeSoftmax, 32, 5>::kSmemBytes;
+  // the list length takes no shared memory in this orientation
+  if (bn == 16) return TcCfg<16, true, kModeSoftmax, 16, 6>::kSmemBytes;
+  if (bn == 32) return TcCfg<32, true, kModeSoftmax, 16, 5>::kSmemBytes;
+  if (bn == 64) return TcCfg<64, true, kModeSoftmax, 16, 5>::kSmemBytes;
+  if (bn == 128) return TcCfg<128, true, kModeSoftmax, 16, 4>::kSmemBytes;
   return 0;
 }
 
