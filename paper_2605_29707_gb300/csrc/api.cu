@@ -84,9 +84,9 @@ struct Plan {
   int num_sms;
   // fused vocabulary GEMM
   bool swap;
-  int bn, kmax, rec, tok_tiles, w_tiles, nchunks, w_per_chunk, grid;
+  int bn, kmax, rec, tok_tiles, w_tiles, nchunks, w_per_chunk, rows_chunk, tail_rows, grid;
   StorePlan xg, ug;
-  int mcast;   // vocab GEMM, tokens on M: CTAs per cluster sharing each weight box (1 = off)
+  bool pair;   // vocab GEMM, tokens on M in an even number of tiles: CTA pairs
   bool chain;  // head kernels launched as a programmatic-dependent chain (small M with overlap)
   bool fused;  // chain path whose GRU computes E . W_ih^T and hidden . W1[:, :H] itself (no
                // gather and no projection GEMMs; the step's first kernel is the GRU)
@@ -163,7 +163,9 @@ int check_sizes(int B, int K, int H, int V, int Ds, int R, int k, int N, bool he
 }
 
 // The plan for a GPU with `sms` SMs (sizes already checked).
-int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool head, int sms, Plan* P) {
+// even_chunks: see the split of the vocabulary below.
+int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool head, int sms, Plan* P,
+                  bool even_chunks = true) {
   Plan& p = *P;
   p = Plan{};  // every member zero (the nested plans' defaults are zero too)
   p.B = B; p.K = K; p.H = H; p.V = V; p.k = k; p.N = N;
@@ -182,13 +184,22 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
   p.w_tiles = p.swap ? ceil_div(V, 128) : ceil_div(V, p.bn);
   int per_tok = sms / p.tok_tiles;
   if (per_tok < 1) per_tok = 1;
+  // Tokens on M: pairs of CTAs with consecutive token tiles share each weight tile (2-SM MMA).
+  p.pair = !p.swap && p.tok_tiles % 2 == 0;
+  // Each CTA streams a contiguous chunk of the vocabulary in tiles of 128 (256) rows.  Up to 128
+  // positions, where the launch is bound by HBM, whole tiles would leave the longest chunk up to one
+  // tile above the average (V = 151936, 152 CTAs: eight tiles against 7.81), and the launch takes as
+  // long as its longest chunk; so the chunks are made equal to within the operand's eight rows and
+  // the last tile of each is shorter (B = 1, H = 4096: 217.8 -> 214.3 us a step; B = 2 225.8 -> 220.5).
   p.w_per_chunk = ceil_div(p.w_tiles, per_tok);
-  p.nchunks = ceil_div(p.w_tiles, p.w_per_chunk);
+  p.rows_chunk = p.w_per_chunk * (p.swap ? 128 : p.bn);
+  if (even_chunks && p.swap && p.w_per_chunk > 1) {
+    p.rows_chunk = ceil_div(ceil_div(V, per_tok), 8) * 8;
+    p.w_per_chunk = ceil_div(p.rows_chunk, 128);
+  }
+  p.tail_rows = p.rows_chunk - (p.w_per_chunk - 1) * (p.swap ? 128 : p.bn);
+  p.nchunks = ceil_div(V, p.rows_chunk);
   p.grid = p.tok_tiles * p.nchunks;
-  // Tokens on M: pairs of CTAs with consecutive token tiles of one vocabulary chunk share each
-  // weight box by TMA multicast (halving the weight traffic from L2; clusters of two still
-  // cover every SM).
-  p.mcast = (!p.swap && p.tok_tiles % 2 == 0) ? 2 : 1;
 
   if (head) {
     p.u_in_gru = p.swap;
@@ -273,14 +284,20 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
   return DOMINO_OK;
 }
 
-int make_plan(int B, int K, int H, int V, int Ds, int R, int k, int N, bool head, Plan* P) {
+// The plan for a workspace of `have` bytes (0: as many as it takes).  Equal chunks are a few more than
+// whole-tile ones and so have a few more partial records; where only the latter's fit, they are taken.
+int make_plan(int B, int K, int H, int V, int Ds, int R, int k, int N, bool head, Plan* P, size_t have = 0,
+              bool host = false) {
   int rc = check_sizes(B, K, H, V, Ds, R, k, N, head);
   if (rc != DOMINO_OK) return rc;
   int sms = 0, major = 0, minor = 0;
   rc = device_sms(&sms, &major, &minor);
   if (rc != DOMINO_OK) return rc;
   if (major != 10 || minor != 3) return DOMINO_ERR_UNSUPPORTED;
-  return make_plan_sms(B, K, H, V, Ds, R, k, N, head, sms, P);
+  rc = make_plan_sms(B, K, H, V, Ds, R, k, N, head, sms, P);
+  if (rc == DOMINO_OK && have && (host ? P->host_total : P->dev_total) > have)
+    rc = make_plan_sms(B, K, H, V, Ds, R, k, N, head, sms, P, false);
+  return rc;
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -316,12 +333,11 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t rows, u
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // Maps for one GEMM: activations X [M, inner] (row stride xs) and weights W [rows_w, inner]
-// (row stride ws), in A/B order for the orientation.  With weight multicast (tokens on M) each
-// CTA of a cluster loads 1/mcast of the weight box, so that map's box is bn / mcast rows high.
+// (row stride ws), in A/B order for the orientation; weight boxes w_box rows high (0: a whole tile).
 bool gemm_maps(CUtensorMap* a, CUtensorMap* b, bool swap, int bn, const void* X, int M, int inner, int xs,
-               const void* W, int rows_w, int ws, int mcast = 1) {
-  if (swap) return make_map(a, W, inner, rows_w, ws, 128) && make_map(b, X, inner, M, xs, bn);
-  return make_map(a, X, inner, M, xs, 128) && make_map(b, W, inner, rows_w, ws, bn / (mcast > 1 ? mcast : 1));
+               const void* W, int rows_w, int ws, int w_box = 0) {
+  if (swap) return make_map(a, W, inner, rows_w, ws, w_box ? w_box : 128) && make_map(b, X, inner, M, xs, bn);
+  return make_map(a, X, inner, M, xs, 128) && make_map(b, W, inner, rows_w, ws, w_box ? w_box : bn);
 }
 
 int cuda_rc(cudaError_t e) { return e == cudaSuccess ? DOMINO_OK : DOMINO_ERR_CUDA; }
@@ -574,29 +590,36 @@ int run_step_launches(const Plan& P, const void* hidden, const int32_t* ids, con
   {
     const dm::TcParams base{};
     TcParams tp = base;
-    CUtensorMap maps[4];
-    if (!gemm_maps(&maps[0], &maps[1], P.swap, P.bn, hidden, M, H, H, w_lm, V, H, P.mcast)) return DOMINO_ERR_CUDA;
+    CUtensorMap maps[6];
+    const int box = P.pair ? P.bn / 2 : 0;
+    if (!gemm_maps(&maps[0], &maps[1], P.swap, P.bn, hidden, M, H, H, w_lm, V, H, box) ||
+        !make_map(&maps[4], w_lm, H, V, H, P.tail_rows))
+      return DOMINO_ERR_CUDA;
     if (P.head) {
-      if (!gemm_maps(&maps[2], &maps[3], P.swap, P.bn, u, M, R, R, hw->w2, V, R, P.mcast)) return DOMINO_ERR_CUDA;
+      if (!gemm_maps(&maps[2], &maps[3], P.swap, P.bn, u, M, R, R, hw->w2, V, R, box) ||
+          !make_map(&maps[5], hw->w2, R, V, R, P.tail_rows))
+        return DOMINO_ERR_CUDA;
     } else {
       maps[2] = maps[0];
       maps[3] = maps[1];
+      maps[5] = maps[4];
     }
     tp.nkb1 = ceil_div(H, 64);
     tp.nkb2 = P.head ? ceil_div(R, 64) : 0;
     tp.rows_tok = M; tp.rows_w = V;
     tp.tok_tiles = P.tok_tiles; tp.w_tiles = P.w_tiles;
     tp.nchunks = P.nchunks; tp.w_per_chunk = P.w_per_chunk;
+    tp.rows_chunk = P.rows_chunk; tp.tail_rows = P.tail_rows;
     tp.w_evict_first = P.tok_tiles == 1 ? 1 : 0;
     tp.defer = P.overlap ? P.defer_tiles : 0;
-    tp.mcast = P.mcast;
+    tp.pair = P.pair ? 1 : 0;
     tp.tmem_cols = P.tmem_cols;
     tp.bias = hw ? static_cast<const __nv_bfloat16*>(hw->b2) : nullptr;
     tp.out = reinterpret_cast<float*>(ws + P.off_part);
     tp.status = status;
     // large M on CTA pairs: a programmatic dependent of u_finalize, waiting for it only before
     // the W2 segment (the first tile's W_lm segment streams meanwhile)
-    if (P.head && !P.u_in_gru && !P.swap && P.mcast == 2) tp.pdl_wait = 3;
+    if (P.head && !P.u_in_gru && P.pair) tp.pdl_wait = 3;
     ts = timing_open(DOMINO_KERNEL_VOCAB, st);
     if (P.overlap)
       rc = cuda_rc(dm::launch_tc_softmax_deferred(P.bn, P.kmax, maps, tp, P.grid, st));
@@ -679,7 +702,7 @@ int domino_draft_step(const void* hidden, const int32_t* prefix_ids, const void*
   int rc = check_pointers(hidden, prefix_ids, w_lm, head, hd);
   if (rc) return rc;
   Plan P;
-  rc = make_plan(B, K, H, V, hd ? head->Ds : 0, hd ? head->R : 0, k, N, hd, &P);
+  rc = make_plan(B, K, H, V, hd ? head->Ds : 0, hd ? head->R : 0, k, N, hd, &P, workspace_bytes);
   if (rc) return rc;
   if (workspace_bytes < P.dev_total) return DOMINO_ERR_INVALID_ARG;
   return run_step(P, hidden, prefix_ids, w_lm, head, topk_ids, topk_logp, tree_parent, tree_token, tree_depth,
@@ -697,7 +720,7 @@ int domino_draft_step_host(const void* hidden_host, const int32_t* prefix_ids_ho
     return DOMINO_ERR_INVALID_ARG;
   if ((reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) != 0) return DOMINO_ERR_INVALID_ARG;
   Plan P;
-  int rc = make_plan(B, K, H, V, hd ? head->Ds : 0, hd ? head->R : 0, k, N, hd, &P);
+  int rc = make_plan(B, K, H, V, hd ? head->Ds : 0, hd ? head->R : 0, k, N, hd, &P, workspace_bytes, true);
   if (rc) return rc;
   if (workspace_bytes < P.host_total) return DOMINO_ERR_INVALID_ARG;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -1174,7 +1197,7 @@ extern "C" int domino_draft_step_static_scratch(const void* hidden, const int32_
   int rc = check_pointers(hidden, prefix_ids, w_lm, head, hd);
   if (rc) return rc;
   Plan P;
-  rc = make_plan(B, K, H, V, hd ? head->Ds : 0, hd ? head->R : 0, k, N, hd, &P);
+  rc = make_plan(B, K, H, V, hd ? head->Ds : 0, hd ? head->R : 0, k, N, hd, &P, DOMINO_STATIC_SCRATCH_BYTES);
   if (rc) return rc;
   if (P.dev_total > DOMINO_STATIC_SCRATCH_BYTES) return DOMINO_ERR_UNSUPPORTED;
   void* scratch = nullptr;

@@ -30,9 +30,10 @@ struct TcParams {
   int nkb1, nkb2;
   int rows_tok, rows_w;
   int tok_tiles, w_tiles;
-  // softmax mode: CTA c handles token tile c % tok_tiles and weight tiles
-  // [chunk * w_per_chunk, ...) with chunk = c / tok_tiles
-  int nchunks, w_per_chunk;
+  // softmax mode: CTA c handles token tile c % tok_tiles and the rows_chunk weight rows from
+  // chunk * rows_chunk on, chunk = c / tok_tiles, in w_per_chunk tiles of which, in the swap
+  // orientation, the last has tail_rows rows (its own tensor maps: boxes of that height)
+  int nchunks, w_per_chunk, rows_chunk, tail_rows;
   // store mode: items (tok tile, w tile, split) round-robin over the CTAs
   int splits, kb_per_split, total_items;
   int w_evict_first;
@@ -41,9 +42,8 @@ struct TcParams {
   int pdl_wait;   // launched as a programmatic dependent: 1 = wait for the preceding grid before
                   // the first load, 2 = after the last load, 3 = before the first load of the
                   // second K segment (the pair kernel; 0 = no wait)
-  int mcast;      // tokens-on-M orientation: CTAs per cluster sharing each weight box by TMA
-                  // multicast (1 = off; 2 or 4, dividing tok_tiles); the weight maps' box is
-                  // BN / mcast rows high
+  int pair;       // softmax, tokens on M in an even number of tiles: CTA pairs (tc_pair.cuh); the weight
+                  // maps' boxes are half a tile high
   int tmem_cols;  // TMEM columns to allocate (power of two, 32..512)
   const __nv_bfloat16* bias;  // softmax: b2 [V] or nullptr
   float* out;                 // softmax: partial records [M][rec fields][nchunks]; store: [splits][M][ld_out]
@@ -53,7 +53,8 @@ struct TcParams {
 
 constexpr int kSoftmaxRecWords(int kmax) { return 2 + 2 * kmax; }
 
-// Tensor maps in the order A1, B1, A2, B2 (A = 128-row operand, B = N-row operand).
+// Tensor maps in the order A1, B1, A2, B2 (A = 128-row operand, B = N-row operand), then, in softmax
+// mode with swap, those of the weights' last tile (segment 1, segment 2).
 cudaError_t launch_tc_gemm(int mode, int bn, bool swap, int kmax, const CUtensorMap* maps,
                            const TcParams& p, int grid, cudaStream_t stream);
 // The store-mode GEMM for many tokens (bn 256, tokens on M) launched as a programmatic dependent
@@ -71,8 +72,8 @@ cudaError_t launch_tc_softmax_k8(int bn, bool swap, const CUtensorMap* maps, con
 cudaError_t launch_tc_softmax_deferred_k8(int bn, const CUtensorMap* maps, const TcParams& p, int grid,
                                           cudaStream_t stream);
 int tc_softmax_deferred_smem_k8(int bn);
-// Tokens on M in CTA pairs (mcast = 2, bn 256): the 2-SM MMA variant (tc_pair.cuh); the maps are
-// the same as for the multicast kernel (weight boxes 128 rows high).
+// Tokens on M in CTA pairs (p.pair, bn 256): the 2-SM MMA variant (tc_pair.cuh); the
+// weight boxes are 128 rows high.
 cudaError_t launch_tc_vocab_pair(int kmax, const CUtensorMap* maps, const TcParams& p, int grid, cudaStream_t stream);
 cudaError_t launch_tc_vocab_pair_k8(const CUtensorMap* maps, const TcParams& p, int grid, cudaStream_t stream);
 // Small-M (swap, bn 16..128) store-mode GEMM with four pipeline stages, launched as a

@@ -59,17 +59,31 @@ struct TcCfg {
 
 struct TcItem {
   int tok, w, kb0, kb1, split;
+  int row0, rows;  // with swap: the tile's weight rows
+  bool tail;       // softmax mode with swap: the chunk's last tile
 };
 
-template <int MODE>
+// TILE: weight rows of a tile.  EVEN: equal chunks, whose last tile is shorter (weights
+// on the 128-row operand; with weights on N the launch is bound by the tensor cores, where equal
+// chunks gained under 1 % and the code for them cost up to 6 %; the loop's store-mode GEMM over the
+// vocabulary, whose CTAs take its tiles in turn, lost 2 % to them at B = 4).
+template <int MODE, int TILE, bool EVEN>
 __device__ __forceinline__ bool tc_get_item(const TcParams& p, int i, TcItem& it) {
   const int nkb = p.nkb1 + p.nkb2;
   if (MODE == kModeSoftmax) {
     const int tok = blockIdx.x % p.tok_tiles;
     const int chunk = blockIdx.x / p.tok_tiles;
-    const int w = chunk * p.w_per_chunk + i;
-    if (chunk >= p.nchunks || i >= p.w_per_chunk || w >= p.w_tiles) return false;
-    it.tok = tok; it.w = w; it.kb0 = 0; it.kb1 = nkb; it.split = 0;
+    it.tok = tok; it.kb0 = 0; it.kb1 = nkb; it.split = 0;
+    if constexpr (EVEN) {
+      it.row0 = chunk * p.rows_chunk + i * TILE;
+      if (chunk >= p.nchunks || i >= p.w_per_chunk || it.row0 >= p.rows_w) return false;
+      it.tail = i == p.w_per_chunk - 1;
+      it.rows = it.tail ? p.tail_rows : TILE;
+    } else {
+      const int w = chunk * p.w_per_chunk + i;
+      if (chunk >= p.nchunks || i >= p.w_per_chunk || w >= p.w_tiles) return false;
+      it.w = w;
+    }
     return true;
   } else {
     const int idx = blockIdx.x + i * gridDim.x;
@@ -81,6 +95,7 @@ __device__ __forceinline__ bool tc_get_item(const TcParams& p, int i, TcItem& it
     it.split = split;
     it.kb0 = split * p.kb_per_split;
     it.kb1 = min(nkb, it.kb0 + p.kb_per_split);
+    it.row0 = it.w * TILE;
     return true;
   }
 }
@@ -253,8 +268,10 @@ template <int BN, bool SWAP, int MODE, int KMAX, int ST>
 __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
                    const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
+                   const __grid_constant__ CUtensorMap tmT1, const __grid_constant__ CUtensorMap tmT2,
                    const TcParams p) {
   using C = TcCfg<BN, SWAP, MODE, KMAX, ST>;
+  constexpr int kTile = SWAP ? 128 : BN;  // weight rows of a tile
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -277,7 +294,7 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], p.mcast > 1 ? p.mcast : 1);  // every CTA of a multicast cluster releases it
+      mbar_init(&empty[s], 1);
     }
     for (int a = 0; a < tc_blocks<BN>(p); ++a) {
       mbar_init(&tfull[a], 1);
@@ -294,6 +311,10 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
       tma_prefetch_desc(&tmA2);
       tma_prefetch_desc(&tmB2);
     }
+    if (MODE == kModeSoftmax && SWAP) {
+      tma_prefetch_desc(&tmT1);
+      if (p.nkb2 > 0) tma_prefetch_desc(&tmT2);
+    }
   }
   if (warp == 1) {
     tmem_alloc(tmem_slot, static_cast<uint32_t>(p.tmem_cols));
@@ -303,12 +324,6 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // Weight multicast (p.mcast > 1, tokens-on-M orientation): the CTAs of a cluster hold
-  // consecutive token tiles of one vocabulary chunk and stream the same weight tiles; each loads
-  // 1/mcast of every weight box into all of them.  No CTA may multicast before every CTA of the
-  // cluster has initialised its barriers.
-  const uint16_t mc_mask = static_cast<uint16_t>((1u << (p.mcast > 1 ? p.mcast : 1)) - 1u);
-  if (p.mcast > 1) cluster_sync();
   // A kernel launched as this grid's programmatic dependent may start now: it waits for this
   // grid to complete before it reads anything this kernel writes.  The trigger comes after the
   // TMEM allocation, so a dependent that allocates TMEM on this SM can only wait for columns
@@ -337,27 +352,23 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
       const int passes = p.defer ? 3 : 1;
       for (int pass = 0; pass < passes && ok; ++pass) {
       if (pass == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
-      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE>(p, i, it); ++i) {
+      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE, kTile, SWAP>(p, i, it); ++i) {
         if (pass < 2 && p.defer && i >= p.defer) break;
         const int kb_lo = (p.defer && pass == 1) ? p.nkb1 : it.kb0;
         const int kb_hi = (p.defer && pass == 0) ? p.nkb1 : it.kb1;
         for (int kb = kb_lo; kb < kb_hi; ++kb) {
           if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
-          mbar_arrive_expect_tx(&full[stage], C::kStageBytes);
+          const bool tail = MODE == kModeSoftmax && SWAP && it.tail;  // fewer weight rows, by their own maps
+          mbar_arrive_expect_tx(&full[stage], tail ? C::kBBytes + it.rows * 128 : C::kStageBytes);
           const bool seg2 = kb >= p.nkb1;
           const int kx = (seg2 ? kb - p.nkb1 : kb) * 64;
-          const int ay = SWAP ? it.w * 128 : it.tok * 128;
+          const int ay = SWAP ? it.row0 : it.tok * 128;
           const int by = SWAP ? it.tok * BN : it.w * BN;
-          tma_load_2d(sA + stage * C::kABytes, seg2 ? &tmA2 : &tmA1, &full[stage], kx, ay, polA);
-          if (!SWAP && p.mcast > 1) {
-            // this CTA's BN / mcast rows of the weight box (the map's box is that high)
-            const int part = static_cast<int>(cluster_ctarank());
-            const int rows = BN / p.mcast;
-            tma_load_2d_multicast(sB + stage * C::kBBytes + part * rows * 128, seg2 ? &tmB2 : &tmB1, &full[stage],
-                                  kx, by + part * rows, mc_mask, polB);
-          } else {
-            tma_load_2d(sB + stage * C::kBBytes, seg2 ? &tmB2 : &tmB1, &full[stage], kx, by, polB);
-          }
+          const CUtensorMap* mw = tail ? (seg2 ? &tmT2 : &tmT1)
+                                       : (SWAP ? (seg2 ? &tmA2 : &tmA1) : (seg2 ? &tmB2 : &tmB1));
+          const CUtensorMap* mt = SWAP ? (seg2 ? &tmB2 : &tmB1) : (seg2 ? &tmA2 : &tmA1);
+          tma_load_2d(sA + stage * C::kABytes, SWAP ? mw : mt, &full[stage], kx, ay, polA);
+          tma_load_2d(sB + stage * C::kBBytes, SWAP ? mt : mw, &full[stage], kx, by, polB);
           ++issued;
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
         }
@@ -365,16 +376,14 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
       }
       if (p.pdl_wait == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
       // Let every load this thread issued land before the CTA can exit (each is the last
-      // one on its stage; a completed phase of that parity returns at once).  With multicast,
-      // wait until every CTA of the cluster has consumed them (the stage's release).
+      // one on its stage; a completed phase of that parity returns at once).
       const int outstanding = issued < C::kStages ? issued : C::kStages;
       for (int j = 1; j <= outstanding; ++j) {
         int s = stage - j;
         uint32_t ph = phase;
         if (s < 0) { s += C::kStages; ph ^= 1u; }
-        uint64_t* last = p.mcast > 1 ? &empty[s] : &full[s];
         const long long t0 = clock64();
-        while (!mbar_try_wait(last, ph)) {
+        while (!mbar_try_wait(&full[s], ph)) {
           if (clock64() - t0 > kWaitCycles) { set_status(p.status, kStatusTimeout); break; }
         }
       }
@@ -389,13 +398,15 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
       TcItem it;
       const int passes = p.defer ? 3 : 1;
       for (int pass = 0; pass < passes && ok; ++pass) {
-      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE>(p, i, it); ++i) {
+      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE, kTile, SWAP>(p, i, it); ++i) {
         if (pass < 2 && p.defer && i >= p.defer) break;
         // a deferred tile (i < p.defer <= blocks) is its block's first; a block used before waits
         // for the epilogue of the tile it held
         const int nblk = tc_blocks<BN>(p), ab = i & (nblk - 1);
         const bool last_pass = !p.defer || pass >= 1;  // passes that finish a tile
         const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ab * BN);
+        // (the rows a shorter last tile lacks hold whatever the stage held; the epilogue skips their
+        // accumulator lanes)
         if (i >= nblk) {
           if (!mbar_wait(&tempty[ab], (i / nblk - 1) & 1, abort_flag, p.status)) break;
           tc_fence_after();
@@ -412,8 +423,7 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
             tc_mma_bf16(d_tmem, da + static_cast<uint64_t>(2 * kk), db + static_cast<uint64_t>(2 * kk),
                         kIdesc, (kb > it.kb0 || kk > 0) ? 1u : 0u);
           }
-          if (p.mcast > 1) tc_commit_multicast(&empty[stage], mc_mask);  // release it in every CTA
-          else tc_commit(&empty[stage]);
+          tc_commit(&empty[stage]);
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
         }
         if (ok && last_pass) tc_commit(&tfull[ab]);
@@ -431,7 +441,7 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
     bool aborted = false;
     TcItem it;
     it.tok = 0;
-    for (int i = 0; tc_get_item<MODE>(p, i, it); ++i) {
+    for (int i = 0; tc_get_item<MODE, kTile, SWAP>(p, i, it); ++i) {
       const int nblk = tc_blocks<BN>(p), ab = i & (nblk - 1);
       const bool ok = mbar_wait(&tfull[ab], (i / nblk) & 1, abort_flag, p.status);
       if (epi_any(!ok)) { aborted = true; break; }
@@ -440,7 +450,7 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
 
       if constexpr (MODE == kModeStore) {
         if constexpr (SWAP) {
-          const int n = it.w * 128 + 32 * q + lane;
+          const int n = it.row0 + 32 * q + lane;
           float* out = p.out + static_cast<size_t>(it.split) * p.rows_tok * p.ld_out;
 #pragma unroll
           for (int c0 = 0; c0 < BN; c0 += (BN < 32 ? BN : 32)) {
@@ -481,8 +491,9 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
         // vocabulary rows on TMEM lanes, tokens on columns: stage kTrRows rows at a time through
         // shared memory so that each thread owns one token and a strided slice of the rows
         const int vrow = 32 * q + lane;
-        const int v = it.w * 128 + vrow;
-        const bool vvalid = v < p.rows_w;
+        const int v = it.row0 + vrow;
+        const int vend = min(p.rows_w, it.row0 + it.rows);
+        const bool vvalid = v < vend;
         const float bv = (p.bias != nullptr && vvalid) ? __bfloat162float(p.bias[v]) : 0.f;
         const int tt = ep / C::kTPT;
         const int sub = ep % C::kTPT;
@@ -503,8 +514,8 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
             mbar_arrive(&tempty[ab]);
           }
           named_bar_sync(1, 128);
-          const int vbase = it.w * 128 + h0 + sub;
-          const int left = p.rows_w - vbase;  // valid entries: vbase + TPT * j < rows_w
+          const int vbase = it.row0 + h0 + sub;
+          const int left = vend - vbase;  // valid entries: vbase + TPT * j < vend
           const int nvalid = left <= 0 ? 0 : (left + C::kTPT - 1) / C::kTPT;
           float r[kSub];
 #pragma unroll
@@ -564,7 +575,6 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
   // ------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
-  if (p.mcast > 1) cluster_sync();  // no CTA leaves while a peer may still write into it
   if (warp == 1) {
     if (lane == 0) {
       // every MMA this thread issued must be finished before the TMEM is released
@@ -597,22 +607,10 @@ cudaError_t launch_tc_instance(const CUtensorMap* maps, const TcParams& p, int g
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchAttribute attrs[2];
-  int na = 0;
-  if (pdl) attrs[na++] = attr[0];
-  if (p.mcast > 1) {
-    if (SWAP || MODE != kModeSoftmax || p.mcast > 8 || p.tok_tiles % p.mcast != 0 || grid % p.mcast != 0 ||
-        BN % (8 * p.mcast) != 0)
-      return cudaErrorInvalidValue;
-    attrs[na].id = cudaLaunchAttributeClusterDimension;
-    attrs[na].val.clusterDim.x = p.mcast;
-    attrs[na].val.clusterDim.y = 1;
-    attrs[na].val.clusterDim.z = 1;
-    ++na;
-  }
-  cfg.attrs = attrs;
-  cfg.numAttrs = na;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], maps[3], p);
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  constexpr int kT = MODE == kModeSoftmax && SWAP ? 4 : 0;  // no other form reads maps of a last tile
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, maps[0], maps[1], maps[2], maps[3], maps[kT], maps[kT + 1], p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

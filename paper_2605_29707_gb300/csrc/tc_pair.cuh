@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(192, 1)
       bool ok = true;
       bool waited = p.pdl_wait != 3;
       TcItem it;
-      for (int i = 0; ok && tc_get_item<kModeSoftmax>(p, i, it); ++i) {
+      for (int i = 0; ok && tc_get_item<kModeSoftmax, BN, false>(p, i, it); ++i) {
         for (int kb = 0; kb < it.kb1; ++kb) {
           if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
           const bool seg2 = kb >= p.nkb1;
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(192, 1)
       uint32_t phase = 0;
       bool ok = true;
       TcItem it;
-      for (int i = 0; ok && tc_get_item<kModeSoftmax>(p, i, it); ++i) {
+      for (int i = 0; ok && tc_get_item<kModeSoftmax, BN, false>(p, i, it); ++i) {
         const int ab = i & 1;
         const uint32_t aph = (i >> 1) & 1;
         if (!mbar_wait_cluster(&tempty[ab], aph ^ 1u, abort_flag, p.status)) break;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(192, 1)
     bool aborted = false;
     TcItem it;
     it.tok = 0;
-    for (int i = 0; tc_get_item<kModeSoftmax>(p, i, it); ++i) {
+    for (int i = 0; tc_get_item<kModeSoftmax, BN, false>(p, i, it); ++i) {
       const int ab = i & 1;
       const uint32_t aph = (i >> 1) & 1;
       const bool ok = mbar_wait_cluster(&tfull[ab], aph, abort_flag, p.status);
@@ -280,7 +280,7 @@ template <int KMAX>
 cudaError_t launch_tc_vocab_pair_instance(const CUtensorMap* maps, const TcParams& p, int grid, cudaStream_t stream) {
   using C = PairCfg<KMAX>;
   auto kern = tc_vocab_pair_kernel<KMAX>;
-  if (p.mcast != 2 || p.tok_tiles % 2 != 0 || grid % 2 != 0 || p.defer != 0) return cudaErrorInvalidValue;
+  if (p.tok_tiles % 2 != 0 || grid % 2 != 0 || p.defer != 0) return cudaErrorInvalidValue;
   {
     const cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), C::kSmemBytes, true);
     if (e != cudaSuccess) return e;

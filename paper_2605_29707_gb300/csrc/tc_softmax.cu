@@ -14,7 +14,7 @@ cudaError_t launch_tc_vocab_pair(int kmax, const CUtensorMap* maps, const TcPara
 cudaError_t launch_tc_softmax(int bn, bool swap, int kmax, const CUtensorMap* maps, const TcParams& p,
                               int grid, cudaStream_t s) {
   // tokens on M in CTA pairs: the 2-SM MMA kernel (tc_pair.cuh)
-  if (!swap && bn == 256 && p.mcast == 2) return launch_tc_vocab_pair(kmax, maps, p, grid, s);
+  if (!swap && bn == 256 && p.pair) return launch_tc_vocab_pair(kmax, maps, p, grid, s);
   if (kmax == 8) return launch_tc_softmax_k8(bn, swap, maps, p, grid, s);
 #define DM_SM(BN, SW, KM)                                                              \
   if (bn == BN && swap == SW && kmax == KM)                                            \
