@@ -81,6 +81,32 @@ __device__ __forceinline__ bool poll_v4(const uint32_t* p, uint4& v, uint32_t ta
   }
 }
 
+// Packed states (wide launches, whose state rows arrive cleared): eight bf16 values in 16 bytes, each
+// with bit 14 set once it is written.  A state is a convex combination of tanh values, so |h| <= 1
+// and that exponent bit is free; NaN (0x7FC0) reads back as NaN because no |h| <= 1 has a code above
+// 0x3F80 below the bit.  Half the bytes of tagged words: what a step reads from L2 is what bounds it
+// at 16 and more sequences a CTA.
+__device__ __forceinline__ uint16_t packed_state(float h) {
+  return static_cast<uint16_t>(__bfloat16_as_ushort(__float2bfloat16_rn(h)) | 0x4000u);
+}
+__device__ __forceinline__ bool all_written(const uint4& v) {
+  return (v.x & v.y & v.z & v.w & 0x40004000u) == 0x40004000u;
+}
+__device__ __forceinline__ uint32_t unpack_states(uint32_t x) {  // two values: bit 14 back to the value's own
+  const uint32_t y = (x & 0x3FFF3FFFu) + 0x007F007Fu;             // bit 14 of y: above 0x3F80, so NaN
+  return (x & 0xBFFFBFFFu) | (y & 0x40004000u);
+}
+// Reads eight packed states, re-reading until all are written (bounded as poll_v4).
+__device__ __forceinline__ bool poll_packed(const uint16_t* p, uint4& v) {
+  const long long t0 = clock64();
+  while (true) {
+    v = ld_relaxed_v4(reinterpret_cast<const uint32_t*>(p));
+    if (all_written(v)) return true;
+    if (clock64() - t0 > kWaitCycles) return false;
+    if (DOMINO_GRU_BACKOFF_NS > 0) __nanosleep(DOMINO_GRU_BACKOFF_NS);
+  }
+}
+
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -347,7 +373,7 @@ __device__ void fused_projections(const GruParams& p, int j0, int Uc, int b0, in
 // `wstride` elements apart: the tagged states are polled (other CTAs may still be publishing their
 // last step).  A lane takes 8 columns of every 256 in increasing order.  False on a timeout, the
 // same in every lane.
-template <int NM, int NQ>
+template <int NM, int NQ, bool kPacked>
 __device__ __forceinline__ bool u_dots(const GruParams& p, const __nv_bfloat16* w, int wstride, int m0, int nm,
                                        uint32_t tag, int lane, float (&acc)[NM][NQ]) {
   const int Ds = p.Ds;
@@ -364,13 +390,18 @@ __device__ __forceinline__ bool u_dots(const GruParams& p, const __nv_bfloat16* 
 #pragma unroll 1
     for (int r = 0; r < nm; ++r) {
       const uint32_t* srow = p.hx + static_cast<size_t>(m0 + r) * Ds;
-      uint4 sv[8];
+      const uint16_t* prow = reinterpret_cast<const uint16_t*>(p.hx) + static_cast<size_t>(m0 + r) * Ds;
+      uint4 sv[kPacked ? 4 : 8];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {  // issue every load of this slice first
         const int c = c0 + lane * 8 + k * 256;
         if (c < Ds) {
-          sv[2 * k] = ld_relaxed_v4(srow + c);
-          sv[2 * k + 1] = ld_relaxed_v4(srow + c + 4);
+          if constexpr (kPacked) {
+            sv[k] = ld_relaxed_v4(reinterpret_cast<const uint32_t*>(prow + c));
+          } else {
+            sv[2 * k] = ld_relaxed_v4(srow + c);
+            sv[2 * k + 1] = ld_relaxed_v4(srow + c + 4);
+          }
         }
       }
       float a[NQ];
@@ -385,19 +416,33 @@ __device__ __forceinline__ bool u_dots(const GruParams& p, const __nv_bfloat16* 
       for (int k = 0; k < 4; ++k) {
         const int c = c0 + lane * 8 + k * 256;
         if (c >= Ds || !got) continue;
+        float hv[8];  // the eight states
+        if constexpr (kPacked) {
+          if (!all_written(sv[k])) got = got && poll_packed(prow + c, sv[k]);
+          const uint32_t x[4] = {unpack_states(sv[k].x), unpack_states(sv[k].y), unpack_states(sv[k].z),
+                                 unpack_states(sv[k].w)};
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
-          if (!all_tagged(sv[2 * k + h], tag)) got = got && poll_v4(srow + c + 4 * h, sv[2 * k + h], tag);
-        const uint32_t sw[8] = {sv[2 * k].x, sv[2 * k].y, sv[2 * k].z, sv[2 * k].w,
-                                sv[2 * k + 1].x, sv[2 * k + 1].y, sv[2 * k + 1].z, sv[2 * k + 1].w};
+          for (int q2 = 0; q2 < 4; ++q2) {
+            hv[2 * q2] = __uint_as_float(x[q2] << 16);
+            hv[2 * q2 + 1] = __uint_as_float(x[q2] & 0xFFFF0000u);
+          }
+        } else {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            if (!all_tagged(sv[2 * k + h], tag)) got = got && poll_v4(srow + c + 4 * h, sv[2 * k + h], tag);
+          const uint32_t sw[8] = {sv[2 * k].x, sv[2 * k].y, sv[2 * k].z, sv[2 * k].w,
+                                  sv[2 * k + 1].x, sv[2 * k + 1].y, sv[2 * k + 1].z, sv[2 * k + 1].w};
+#pragma unroll
+          for (int q2 = 0; q2 < 8; ++q2) hv[q2] = __uint_as_float(sw[q2] & 0xFFFF0000u);
+        }
 #pragma unroll
         for (int i = 0; i < NQ; ++i) {
           const __nv_bfloat162* w2 = reinterpret_cast<const __nv_bfloat162*>(&wv[i][k]);
 #pragma unroll
           for (int q2 = 0; q2 < 4; ++q2) {
             const float2 wf = __bfloat1622float2(w2[q2]);
-            a[i] = fmaf(wf.x, __uint_as_float(sw[2 * q2] & 0xFFFF0000u), a[i]);
-            a[i] = fmaf(wf.y, __uint_as_float(sw[2 * q2 + 1] & 0xFFFF0000u), a[i]);
+            a[i] = fmaf(wf.x, hv[2 * q2], a[i]);
+            a[i] = fmaf(wf.y, hv[2 * q2 + 1], a[i]);
           }
         }
       }
@@ -427,7 +472,7 @@ template <bool kTable, int kX>
 __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const GruParams p) {
   constexpr bool kWide = kX > 0;
   constexpr int kPollBatch = kWide ? 16 : 8;  // state loads a lane issues before checking tags
-  constexpr bool kRepoll = !kWide;
+  uint16_t* hxp = reinterpret_cast<uint16_t*>(p.hx);  // packed states (wide)
   extern __shared__ __align__(16) uint8_t gsmem[];
   const int U = p.units, Ds = p.Ds, K = p.K, B = p.B, R = p.R, H = p.H;
   const int M = B * K;
@@ -614,45 +659,74 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
         //      state words, stages them and multiplies them at once, so the tensor work on early
         //      k-ranges overlaps the wait for late writers
         const int kw0 = (nk * warp) / kGruWarps, kw1 = (nk * (warp + 1)) / kGruWarps;
-        const int q0 = kw0 * 4, q1 = min(kw1 * 4, Ds / 4);  // 4-word columns of the range
-        const int ncq = max(0, q1 - q0);
-        const int total = nb * ncq;
+        bool got = true;
         // (every CTA reads the states in the same order: with a starting sequence of its own each,
         // the same lines were no longer asked for together and a step took 7.8 instead of 5.6 us at B = 32)
-        bool got = true;
-        for (int e0 = lane; e0 < total && got; e0 += kPollBatch * 32) {
-          uint4 v[kPollBatch];
+        if constexpr (kWide) {
+          const int q0 = kw0 * 2, ncq = max(0, min(kw1 * 2, Ds / 8) - q0);  // 8-value columns of the range
+          const int total = nb * ncq;
+          for (int e0 = lane; e0 < total && got; e0 += kPollBatch * 32) {
+            uint4 v[kPollBatch];
 #pragma unroll
-          for (int i = 0; i < kPollBatch; ++i) {  // issue every load first, then check the flags
-            const int e = e0 + i * 32;
-            if (e < total) {
-              const size_t m = static_cast<size_t>(b0 + c0 + e / ncq) * K + (t - 1);
-              v[i] = ld_relaxed_v4(p.hx + m * Ds + (q0 + e % ncq) * 4);
+            for (int i = 0; i < kPollBatch; ++i) {  // issue every load first, then check
+              const int e = e0 + i * 32;
+              if (e < total) {
+                const size_t m = static_cast<size_t>(b0 + c0 + e / ncq) * K + (t - 1);
+                v[i] = ld_relaxed_v4(reinterpret_cast<const uint32_t*>(hxp + m * Ds + (q0 + e % ncq) * 8));
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < kPollBatch; ++i) {
+              const int e = e0 + i * 32;
+              if (e < total && got) {
+                const int bb = e / ncq, cq = q0 + e % ncq;
+                if (!all_written(v[i])) {
+                  const size_t m = static_cast<size_t>(b0 + c0 + bb) * K + (t - 1);
+                  got = poll_packed(hxp + m * Ds + cq * 8, v[i]);
+                }
+                *reinterpret_cast<uint4*>(hsm + static_cast<size_t>(bb) * ldw + cq * 8) =
+                    make_uint4(unpack_states(v[i].x), unpack_states(v[i].y), unpack_states(v[i].z), unpack_states(v[i].w));
+              }
             }
           }
+        } else {
+          const int q0 = kw0 * 4, q1 = min(kw1 * 4, Ds / 4);  // 4-word columns of the range
+          const int ncq = max(0, q1 - q0);
+          const int total = nb * ncq;
+          for (int e0 = lane; e0 < total && got; e0 += kPollBatch * 32) {
+            uint4 v[kPollBatch];
 #pragma unroll
-          for (int i = 0; i < kPollBatch; ++i) {
-            const int e = e0 + i * 32;
-            if (e < total && got) {
-              const int bb = e / ncq, cq = q0 + e % ncq;
-              if (!all_tagged(v[i], tag)) {
-                const size_t m = static_cast<size_t>(b0 + c0 + bb) * K + (t - 1);
-                got = poll_v4(p.hx + m * Ds + cq * 4, v[i], tag);
-                // the batch was early: by now its other late words are probably there, so they are
-                // read again together rather than one round trip after another
-                if (kRepoll) {
+            for (int i = 0; i < kPollBatch; ++i) {  // issue every load first, then check the flags
+              const int e = e0 + i * 32;
+              if (e < total) {
+                const size_t m = static_cast<size_t>(b0 + c0 + e / ncq) * K + (t - 1);
+                v[i] = ld_relaxed_v4(p.hx + m * Ds + (q0 + e % ncq) * 4);
+              }
+            }
 #pragma unroll
-                  for (int i2 = 0; i2 < kPollBatch; ++i2) {
-                    const int e2 = e0 + i2 * 32;
-                    if (i2 > i && e2 < total && !all_tagged(v[i2], tag)) {
-                      const size_t m2 = static_cast<size_t>(b0 + c0 + e2 / ncq) * K + (t - 1);
-                      v[i2] = ld_relaxed_v4(p.hx + m2 * Ds + (q0 + e2 % ncq) * 4);
+            for (int i = 0; i < kPollBatch; ++i) {
+              const int e = e0 + i * 32;
+              if (e < total && got) {
+                const int bb = e / ncq, cq = q0 + e % ncq;
+                if (!all_tagged(v[i], tag)) {
+                  const size_t m = static_cast<size_t>(b0 + c0 + bb) * K + (t - 1);
+                  got = poll_v4(p.hx + m * Ds + cq * 4, v[i], tag);
+                  // the batch was early: by now its other late words are probably there, so they are
+                  // read again together rather than one round trip after another
+                  {
+#pragma unroll
+                    for (int i2 = 0; i2 < kPollBatch; ++i2) {
+                      const int e2 = e0 + i2 * 32;
+                      if (i2 > i && e2 < total && !all_tagged(v[i2], tag)) {
+                        const size_t m2 = static_cast<size_t>(b0 + c0 + e2 / ncq) * K + (t - 1);
+                        v[i2] = ld_relaxed_v4(p.hx + m2 * Ds + (q0 + e2 % ncq) * 4);
+                      }
                     }
                   }
                 }
+                *reinterpret_cast<uint2*>(hsm + static_cast<size_t>(bb) * ldw + cq * 4) =
+                    make_uint2(pack_hi_halves(v[i].x, v[i].y), pack_hi_halves(v[i].z, v[i].w));
               }
-              *reinterpret_cast<uint2*>(hsm + static_cast<size_t>(bb) * ldw + cq * 4) =
-                  make_uint2(pack_hi_halves(v[i].x, v[i].y), pack_hi_halves(v[i].z, v[i].w));
             }
           }
         }
@@ -748,7 +822,8 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
         const float h = (1.f - z) * n + z * hp;
         hprev[bl * U + jl] = h;
         if (held && hold.x == kHoldPublish && hold.z == t) continue;  // test hook: withheld
-        p.hx[m * Ds + j] = tagged(h, tag);
+        if (kWide) __stcg(hxp + m * Ds + j, packed_state(h));
+        else p.hx[m * Ds + j] = tagged(h, tag);
         if (p.s_out) p.s_out[m * Ds + j] = __float2bfloat16_rn(h);
       }
       __syncthreads();
@@ -772,7 +847,7 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
       const float bq = bf_or0(p.b1, q);
       for (int m = mg; m < M; m += groups) {
         float acc[1][1] = {{0.f}};
-        if (!u_dots<1, 1>(p, w1row, 0, m, 1, tag, lane, acc)) {
+        if (!u_dots<1, 1, false>(p, w1row, 0, m, 1, tag, lane, acc)) {
           if (lane == 0) set_status(p.status, kStatusTimeout);
           return;
         }
@@ -799,7 +874,7 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
     for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[r][i] = 0.f;
-    if (!u_dots<4, 4>(p, p.w1 + static_cast<size_t>(q0) * (H + Ds) + H, H + Ds, m0, nm, tag, lane, acc)) {
+    if (!u_dots<4, 4, kWide>(p, p.w1 + static_cast<size_t>(q0) * (H + Ds) + H, H + Ds, m0, nm, tag, lane, acc)) {
       if (lane == 0) set_status(p.status, kStatusTimeout);
       return;
     }

@@ -97,7 +97,8 @@ cudaError_t launch_gather(const GatherParams& p, cudaStream_t stream);
 // GRU recurrence.  CTA (cu, cb) of a gu x gb grid owns hidden units [cu*units, cu*units+units)
 // (gate rows r|z|n of each) for sequences [cb*bc, cb*bc+bc).  States travel between CTAs as
 // tagged words in hx: bf16 value in the high half, a non-zero flag in the low half, one row
-// per (sequence, position) written once per step, so a reader polls the data itself.
+// per (sequence, position) written once per step, so a reader polls the data itself; wide launches
+// pack them as 16-bit values with a written bit (gru.cu).
 struct GruParams {
   const float* xpart;  // [xsplits][M][3*Ds]  partial sums of E . W_ih^T
   int xsplits;
