@@ -22,7 +22,7 @@
 namespace dm {
 
 constexpr int kGruThreads = 256;
-constexpr int kGatePairsPerThread = 2;  // (sequence, unit) gate evaluations per thread and chunk
+constexpr int kGatePairsPerThread = 2;  // most (sequence, unit) gate evaluations per thread and chunk
 constexpr int kGruWarps = kGruThreads / 32;
 constexpr int kChunkSeqs = 32;  // sequences staged per MMA pass (4 n-tiles of 8)
 constexpr int kMaxMt = 3;  // 16-row gate tiles per CTA (up to 16 units x 3 gates)
@@ -468,10 +468,13 @@ __device__ __forceinline__ bool u_dots(const GruParams& p, const __nv_bfloat16* 
 // ones are added at the gates): at d_s = 1024 there are at most 3 above 384 positions and 6 below,
 // where holding three, and waiting for the rest before the poll, made a step 6.8 instead of 4.7 us
 // at B = 12; holding six everywhere costs spills (B = 64: 8.7 -> 9.2 us a step).
-template <bool kTable, int kX>
+// kPairs: gate evaluations per thread (1 when a chunk has at most 256, i.e. 16 units x 16 sequences)
+// and, with them, the state loads in flight: what a launch does not need is registers, and a
+// spilled X partial sum is waited for before the poll (B = 32: 5.25 us a step against 4.4).
+template <bool kTable, int kX, int kPairs>
 __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const GruParams p) {
   constexpr bool kWide = kX > 0;
-  constexpr int kPollBatch = kWide ? 16 : 8;  // state loads a lane issues before checking tags
+  constexpr int kPollBatch = kWide ? 8 * kPairs : 8;  // state loads a lane issues before checking them
   uint16_t* hxp = reinterpret_cast<uint16_t*>(p.hx);  // packed states (wide)
   extern __shared__ __align__(16) uint8_t gsmem[];
   const int U = p.units, Ds = p.Ds, K = p.K, B = p.B, R = p.R, H = p.H;
@@ -600,9 +603,9 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
   bool ok = true;
   // The biases of this thread's gate pairs do not change from step to step (pair e of a chunk is
   // unit e % Uc).  b_ih is already in xs except when the steps read a table row or X partials.
-  float bih[kGatePairsPerThread][3], bhh[kGatePairsPerThread][3];
+  float bih[kPairs][3], bhh[kPairs][3];
 #pragma unroll
-  for (int r = 0; r < kGatePairsPerThread; ++r) {
+  for (int r = 0; r < kPairs; ++r) {
     const int j = j0 + (Uc > 0 ? (tid + r * kGruThreads) % Uc : 0);
 #pragma unroll
     for (int g = 0; g < 3; ++g) {
@@ -619,9 +622,9 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
       // gate inputs of this step: issued as loads now and summed only at the gates, after the
       // wait for h_{t-1}, so that no instruction stalls on them before the wait
       constexpr int kXr = kWide ? kX : 1;
-      float gx[kGatePairsPerThread][3][kXr];
+      float gx[kPairs][3][kXr];
 #pragma unroll
-      for (int r = 0; r < kGatePairsPerThread; ++r) {
+      for (int r = 0; r < kPairs; ++r) {
         const int e = tid + r * kGruThreads;
 #pragma unroll
         for (int g = 0; g < 3; ++g)
@@ -683,6 +686,17 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
                 if (!all_written(v[i])) {
                   const size_t m = static_cast<size_t>(b0 + c0 + bb) * K + (t - 1);
                   got = poll_packed(hxp + m * Ds + cq * 8, v[i]);
+                  // the batch was early: by now its other late states are probably there, so they are
+                  // read again together rather than one round trip after another (B = 32: steps of 4.2 to
+                  // 10 us became 4.2; batches of 16 lose to it: 6.0 against 6.35 at B = 64)
+#pragma unroll
+                  for (int i2 = kPairs == 1 ? i + 1 : kPollBatch; i2 < kPollBatch; ++i2) {
+                    const int e2 = e0 + i2 * 32;
+                    if (e2 < total && !all_written(v[i2])) {
+                      const size_t m2 = static_cast<size_t>(b0 + c0 + e2 / ncq) * K + (t - 1);
+                      v[i2] = ld_relaxed_v4(reinterpret_cast<const uint32_t*>(hxp + m2 * Ds + (q0 + e2 % ncq) * 8));
+                    }
+                  }
                 }
                 *reinterpret_cast<uint4*>(hsm + static_cast<size_t>(bb) * ldw + cq * 8) =
                     make_uint4(unpack_states(v[i].x), unpack_states(v[i].y), unpack_states(v[i].z), unpack_states(v[i].w));
@@ -788,7 +802,7 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
       }
       // ---- gates and the new state (torch.nn.GRU convention); publish the tagged state
 #pragma unroll
-      for (int rr = 0; rr < kGatePairsPerThread; ++rr) {
+      for (int rr = 0; rr < kPairs; ++rr) {
         const int e = tid + rr * kGruThreads;
         if (e >= nb * Uc) break;
         const int bb = e / Uc, jl = e % Uc;
@@ -808,8 +822,7 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
           if constexpr (kXr > 1) {  // partial sums 0, 3, 4, ..., then 1 and 2
 #pragma unroll
             for (int q = 3; q < kXr; ++q) s += gx[rr][g][q];
-            if (!kTable)
-              for (int q = kXr; q < p.xsplits; ++q) s += p.xpart[(q * static_cast<size_t>(M) + m) * 3 * Ds + g * Ds + j];
+            for (int q = kXr; q < p.xsplits; ++q) s += p.xpart[(q * static_cast<size_t>(M) + m) * 3 * Ds + g * Ds + j];
             s += gx[rr][g][1];
             s += gx[rr][g][2];
           }
@@ -925,11 +938,11 @@ GruPlan gru_plan(int B, int Ds, int num_sms) {
   return g;
 }
 
-template <bool kTable, int kX>
+template <bool kTable, int kX, int kPairs>
 static cudaError_t launch_gru_t(const GruParams& p, const GruPlan& plan, cudaStream_t stream, bool pdl) {
   {
     const cudaError_t e =
-        ensure_smem_attr(reinterpret_cast<const void*>(gru_kernel<kTable, kX>), plan.smem, true);
+        ensure_smem_attr(reinterpret_cast<const void*>(gru_kernel<kTable, kX, kPairs>), plan.smem, true);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
@@ -946,12 +959,12 @@ static cudaError_t launch_gru_t(const GruParams& p, const GruPlan& plan, cudaStr
   // A runtime that refuses the pair gets the cooperative launch alone from then on.
   static std::atomic<bool> pdl_refused{false};
   cfg.numAttrs = (pdl && !pdl_refused) ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kX>, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kX, kPairs>, p);
   if (e != cudaSuccess && cfg.numAttrs == 2) {
     (void)cudaGetLastError();
     pdl_refused = true;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kX>, p);
+    e = cudaLaunchKernelEx(&cfg, gru_kernel<kTable, kX, kPairs>, p);
   }
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -960,10 +973,23 @@ static cudaError_t launch_gru_t(const GruParams& p, const GruPlan& plan, cudaStr
 cudaError_t launch_gru(const GruParams& p, const GruPlan& plan, cudaStream_t stream, bool pdl, bool wide) {
   if (plan.smem == 0) return cudaErrorInvalidValue;
   if (wide && p.ids != nullptr) return cudaErrorInvalidValue;  // fused projections share SMs
-  if (!wide)
-    return p.x_table ? launch_gru_t<true, 0>(p, plan, stream, pdl) : launch_gru_t<false, 0>(p, plan, stream, pdl);
-  if (p.x_table) return launch_gru_t<true, 1>(p, plan, stream, pdl);
-  return p.xsplits <= 3 ? launch_gru_t<false, 3>(p, plan, stream, pdl) : launch_gru_t<false, 6>(p, plan, stream, pdl);
+  // gate evaluations of a CTA's largest chunk of sequences
+  const int chunk = p.bc < kChunkSeqs ? p.bc : kChunkSeqs;
+  const bool one = chunk * p.units <= kGruThreads;
+  if (!wide) {
+    if (one)
+      return p.x_table ? launch_gru_t<true, 0, 1>(p, plan, stream, pdl) : launch_gru_t<false, 0, 1>(p, plan, stream, pdl);
+    // many short sequences on a small d_s, whose CTAs still fit beside the vocabulary GEMM's
+    return p.x_table ? launch_gru_t<true, 0, 2>(p, plan, stream, pdl) : launch_gru_t<false, 0, 2>(p, plan, stream, pdl);
+  }
+  if (p.x_table)
+    return one ? launch_gru_t<true, 1, 1>(p, plan, stream, pdl) : launch_gru_t<true, 1, 2>(p, plan, stream, pdl);
+  if (one)
+    return p.xsplits <= 3 ? launch_gru_t<false, 3, 1>(p, plan, stream, pdl)
+                          : launch_gru_t<false, 6, 1>(p, plan, stream, pdl);
+  return p.xsplits <= 1   ? launch_gru_t<false, 1, 2>(p, plan, stream, pdl)
+         : p.xsplits <= 3 ? launch_gru_t<false, 3, 2>(p, plan, stream, pdl)
+                          : launch_gru_t<false, 6, 2>(p, plan, stream, pdl);
 }
 
 // ---------------------------------------------------------------------------- u finalize

@@ -15,6 +15,9 @@ CASES = {
     "m64-k10": dict(B=4, K=16, H=128, V=152 * 128 * 3 - 3, Ds=136, R=72, k=10, N=32, seed=82, biases=True),
     "m65": dict(B=5, K=13, H=64, V=152 * 128 * 4 + 100, Ds=64, R=64, k=8, N=9, seed=83),
     "m128-k20": dict(B=8, K=16, H=64, V=152 * 128 * 4 + 1, Ds=256, R=40, k=20, N=24, seed=84, biases=True),
+    # 100 sequences of one position on a small d_s: two gate evaluations a thread beside the vocabulary GEMM
+    "m100-b100": dict(B=100, K=1, H=64, V=3001, Ds=64, R=64, k=4, N=4, seed=86),
+    "m120-b40": dict(B=40, K=3, H=64, V=3001, Ds=64, R=64, k=4, N=8, seed=87, biases=True),
     "m102-ds1032": dict(B=6, K=17, H=64, V=3001, Ds=1032, R=64, k=4, N=12, seed=85),
 }
 
