@@ -197,51 +197,102 @@ __device__ __forceinline__ float f32_from_ord(uint32_t o) {
   return __uint_as_float((o & 0x80000000u) ? (o & 0x7FFFFFFFu) : ~o);
 }
 
-// The best-first tree for N <= 31 (every slot in its own lane's registers): the same selection,
-// keys and tie rules as the general warp version below, with a short dependency chain per pop.
-// The popped child's score and token come out of the winning key itself; only the parent's depth
-// crosses lanes; the two slots that change (the popped one and the new node) each compute their
-// next best child in their own lane, on the same instruction path.
+// The best-first tree for N <= 32: the same selection, keys and tie rules as the general warp version
+// below, with a short dependency chain per pop.  Slot s (the anchor, then node s - 1) lives in lane s's
+// registers; the 32nd node is never expanded and takes the anchor's lane.  The popped child's score
+// and token come out of the winning key itself; only the parent's depth crosses lanes; the two slots
+// that change (the popped one and the new node) each compute their next best child in their own
+// lane, on the same instruction path.
+// While no two children of a slot tie exactly, a slot's taken entries are the head of its row, so its
+// next child is the next entry: one shared-memory round trip, and no second reduction unless two
+// slots' children tie.  The first tie among a slot's children (rare) ends that loop, and the loop on
+// entry masks goes on from the same state.  Bound by that chain (one warp); a pop took 0.31 us with
+// masks throughout, 0.18 so (merge and tree at B = 1, N = 16: 15.9 -> 14.2 us; B = 64, N = 32: 34.9 -> 29.6).
 __device__ void tree_lanes(const float* lp, const int* ids, int K, int k, int N, unsigned all, int lane,
                            int32_t* tpar, int32_t* ttok, int32_t* tdep, float* tsc) {
-  // slot `lane`: score, depth, mask of selected entries, cached best child (hi, lo, j), and the
-  // node it is (parent index, token)
+  // slot `lane`: score, depth, cached best child (hi, lo), and the node it is (parent index, token);
+  // off: the cached child's entry (row * k + index), left: the row's entries from it on
   float score = 0.f;
-  int depth = 0, j = 0, par = -1, tok = -1;
-  unsigned mask = 0u;
+  int depth = 0, par = -1, tok = -1;
+  int off = 0, left = lane == 0 ? k : 0;
   uint32_t hi = 0u, lo = 0u;
-  own_best_child(lp, ids, k, 0, 0.f, lane == 0 ? all : 0u, 0, hi, lo, j);
-  int n_sel = 0;
-  for (int i = 0; i < N; ++i) {
-    const bool live = lane <= i;
-    const uint32_t mhi = __reduce_max_sync(0xffffffffu, live ? hi : 0u);
+  const unsigned slot_lo = 0x3FFu - static_cast<unsigned>(lane);
+  // the child at `off`; true when the next entry ties it exactly
+  auto take = [&]() {
+    const float v = lp[off], v1 = lp[off + (left > 1 ? 1 : 0)];
+    const int id = ids[off];
+    const float s0 = score + v;
+    hi = left > 0 ? f32_ord(s0) : 0u;
+    lo = left > 0 ? ((0x3FFFFFu - static_cast<unsigned>(id)) << 10) | slot_lo : 0u;
+    return left > 1 && score + v1 == s0;
+  };
+  bool tie = lane == 0 && take();
+  int i = 0;
+  bool out = false;
+  if (__any_sync(0xffffffffu, tie)) goto masks;
+  for (; i < N; ++i) {
+    const uint32_t mhi = __reduce_max_sync(0xffffffffu, hi);
     if (mhi == 0u) break;  // no frontier left (the host keeps N within the tree's capacity)
-    const uint32_t mlo = __reduce_max_sync(0xffffffffu, (live && hi == mhi) ? lo : 0u);
-    const int src = __ffs(__ballot_sync(0xffffffffu, live && hi == mhi && lo == mlo)) - 1;
-    const int d = __shfl_sync(0xffffffffu, depth, src);
-    const float sc = f32_from_ord(mhi);
-    const int t = static_cast<int>(0x3FFFFFu - (mlo >> 10));
-    const bool is_new = lane == i + 1, is_src = lane == src;
-    if (is_new) {
-      score = sc;
-      depth = d + 1;
-      mask = 0u;
-      par = src - 1;
-      tok = t;
+    unsigned ball = __ballot_sync(0xffffffffu, hi == mhi);
+    if (ball & (ball - 1u)) {  // several slots' children: the lower token, then the lower slot
+      const uint32_t mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? lo : 0u);
+      ball = __ballot_sync(0xffffffffu, hi == mhi && lo == mlo);
     }
-    if (is_src) mask |= 1u << j;
-    // the two changed slots: the new node's children come from row d + 1 (none past the last
-    // position), the popped slot's from its own row without the entries taken
-    const int row = is_new ? (d + 1 < K ? d + 1 : K - 1) : depth;
-    const unsigned avail = is_new ? (d + 1 < K ? all : 0u) : (~mask & all);
-    if (is_new || is_src) own_best_child(lp, ids, k, row, score, avail, lane, hi, lo, j);
-    n_sel = i + 1;
+    const int src = __ffs(ball) - 1;
+    const int d = __shfl_sync(0xffffffffu, depth, src);
+    const uint32_t l = __shfl_sync(0xffffffffu, lo, src);
+    const bool is_new = lane == ((i + 1) & 31), is_src = lane == src && !is_new;
+    if (is_new) {
+      score = f32_from_ord(mhi);
+      depth = d + 1;
+      par = src - 1;
+      tok = static_cast<int>(0x3FFFFFu - (l >> 10));
+      off = (d + 1 < K ? d + 1 : 0) * k;
+      left = d + 1 < K ? k : 0;
+      out = true;
+    }
+    if (is_src) {
+      ++off;
+      --left;
+      if (left <= 0) off = 0;
+    }
+    tie = (is_new || is_src) && take();
+    if (__any_sync(0xffffffffu, tie)) {
+      ++i;
+      break;
+    }
   }
-  if (lane >= 1 && lane <= n_sel) {  // node lane - 1
-    tpar[lane - 1] = par;
-    ttok[lane - 1] = tok;
-    tdep[lane - 1] = depth;
-    if (tsc) tsc[lane - 1] = score;
+masks:
+  if (__any_sync(0xffffffffu, tie)) {
+    // slot masks: the entries taken are the row's first k - left
+    unsigned mask = left > 0 ? ((1u << (k - left)) - 1u) : all;
+    int j = 0;
+    own_best_child(lp, ids, k, left > 0 ? depth : 0, score, ~mask & all, lane, hi, lo, j);
+    for (; i < N; ++i) {
+      const uint32_t mhi = __reduce_max_sync(0xffffffffu, hi);
+      if (mhi == 0u) break;
+      const uint32_t mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? lo : 0u);
+      const int src = __ffs(__ballot_sync(0xffffffffu, hi == mhi && lo == mlo)) - 1;
+      const int d = __shfl_sync(0xffffffffu, depth, src);
+      const bool is_new = lane == ((i + 1) & 31), is_src = lane == src && !is_new;
+      if (is_src) mask |= 1u << j;
+      if (is_new) {
+        score = f32_from_ord(mhi);
+        depth = d + 1;
+        mask = d + 1 < K ? 0u : all;
+        par = src - 1;
+        tok = static_cast<int>(0x3FFFFFu - (mlo >> 10));
+        out = true;
+      }
+      if (is_new || is_src) own_best_child(lp, ids, k, depth < K ? depth : 0, score, ~mask & all, lane, hi, lo, j);
+    }
+  }
+  if (out) {  // node lane - 1 (the 32nd in lane 0)
+    const int node = (lane + 31) & 31;
+    tpar[node] = par;
+    ttok[node] = tok;
+    tdep[node] = depth;
+    if (tsc) tsc[node] = score;
   }
 }
 
@@ -351,7 +402,7 @@ __global__ void __launch_bounds__(NT, NT == kMergeThreadsNarrow ? 8 : 1) merge_t
   }
   __syncthreads();
   if (warp != 0) return;
-  if (N <= 31) {
+  if (N <= 32) {
     const size_t ob1 = static_cast<size_t>(b) * N;
     tree_lanes(s_lp, s_id, K, k, N, (k == 32) ? 0xffffffffu : ((1u << k) - 1u), lane, p.tree_parent + ob1,
                p.tree_token + ob1, p.tree_depth + ob1, p.tree_score ? p.tree_score + ob1 : nullptr);
