@@ -97,10 +97,10 @@ __device__ __forceinline__ uint32_t unpack_states(uint32_t x) {  // two values: 
   return (x & 0xBFFFBFFFu) | (y & 0x40004000u);
 }
 // Reads eight packed states, re-reading until all are written (bounded as poll_v4).
-__device__ __forceinline__ bool poll_packed(const uint16_t* p, uint4& v) {
+__device__ __forceinline__ bool poll_packed(const uint32_t* p, uint4& v) {
   const long long t0 = clock64();
   while (true) {
-    v = ld_relaxed_v4(reinterpret_cast<const uint32_t*>(p));
+    v = ld_relaxed_v4(p);
     if (all_written(v)) return true;
     if (clock64() - t0 > kWaitCycles) return false;
     if (DOMINO_GRU_BACKOFF_NS > 0) __nanosleep(DOMINO_GRU_BACKOFF_NS);
@@ -418,7 +418,7 @@ __device__ __forceinline__ bool u_dots(const GruParams& p, const __nv_bfloat16* 
         if (c >= Ds || !got) continue;
         float hv[8];  // the eight states
         if constexpr (kPacked) {
-          if (!all_written(sv[k])) got = got && poll_packed(prow + c, sv[k]);
+          if (!all_written(sv[k])) got = got && poll_packed(reinterpret_cast<const uint32_t*>(prow + c), sv[k]);
           const uint32_t x[4] = {unpack_states(sv[k].x), unpack_states(sv[k].y), unpack_states(sv[k].z),
                                  unpack_states(sv[k].w)};
 #pragma unroll
@@ -604,9 +604,12 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
   // The biases of this thread's gate pairs do not change from step to step (pair e of a chunk is
   // unit e % Uc).  b_ih is already in xs except when the steps read a table row or X partials.
   float bih[kPairs][3], bhh[kPairs][3];
+  int pb[kPairs], pj[kPairs];  // a pair's sequence within a chunk and its unit
 #pragma unroll
   for (int r = 0; r < kPairs; ++r) {
-    const int j = j0 + (Uc > 0 ? (tid + r * kGruThreads) % Uc : 0);
+    pb[r] = Uc > 0 ? (tid + r * kGruThreads) / Uc : 0;
+    pj[r] = Uc > 0 ? (tid + r * kGruThreads) % Uc : 0;
+    const int j = j0 + pj[r];
 #pragma unroll
     for (int g = 0; g < 3; ++g) {
       bih[r][g] = (kTable || kWide) ? bf_or0(p.b_ih, g * Ds + j) : 0.f;
@@ -614,6 +617,21 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
     }
   }
 
+  // This warp's k-range of W_hh . h_{t-1} (whole k16 blocks).  Wide: in 16-byte columns of packed states
+  // from q0 on, whose items (sequence, column) go to the lanes in turn: the lane's first, and the way to
+  // its next
+  const int kw0 = (nk * warp) / kGruWarps, kw1 = (nk * (warp + 1)) / kGruWarps;
+  const int q0 = kw0 * 2, ncq = max(0, min(kw1 * 2, Ds / 8) - q0);
+  const int bb0 = ncq > 0 ? lane / ncq : B, cq0 = ncq > 0 ? lane % ncq : 0;
+  const int dq = ncq > 0 ? 32 / ncq : 1, rq = ncq > 0 ? 32 % ncq : 0;
+  auto advance = [&](int& bb, int& cq) {
+    bb += dq;
+    cq += rq;
+    if (cq >= ncq) {
+      cq -= ncq;
+      ++bb;
+    }
+  };
   for (int t = 0; t < K && ok; ++t) {
     for (int c0 = 0; c0 < nbc; c0 += L.chunk) {
       const int nb = min(L.chunk, nbc - c0);
@@ -631,9 +649,8 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
 #pragma unroll
           for (int s = 0; s < kXr; ++s) gx[r][g][s] = 0.f;
         if (e < nb * Uc) {
-          const int bb = e / Uc, jl = e % Uc;
-          const int j = j0 + jl;
-          const size_t m = static_cast<size_t>(b0 + c0 + bb) * K + t;
+          const int j = j0 + pj[r];
+          const size_t m = static_cast<size_t>(b0 + c0 + pb[r]) * K + t;
           // b_ih + W_i{r,z,n} E_m: summed into xs before the steps, or a row of the table (an id
           // outside [0, V), reported by the id check, reads row 0), or the X GEMM's split-K partial
           // sums (wide launches)
@@ -661,46 +678,54 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
         //      of 16 consecutive units, i.e. of one or two writer CTAs): it polls exactly those
         //      state words, stages them and multiplies them at once, so the tensor work on early
         //      k-ranges overlaps the wait for late writers
-        const int kw0 = (nk * warp) / kGruWarps, kw1 = (nk * (warp + 1)) / kGruWarps;
         bool got = true;
         // (every CTA reads the states in the same order: with a starting sequence of its own each,
         // the same lines were no longer asked for together and a step took 7.8 instead of 5.6 us at B = 32)
         if constexpr (kWide) {
-          const int q0 = kw0 * 2, ncq = max(0, min(kw1 * 2, Ds / 8) - q0);  // 8-value columns of the range
-          const int total = nb * ncq;
-          for (int e0 = lane; e0 < total && got; e0 += kPollBatch * 32) {
+          const uint16_t* src = hxp + (static_cast<size_t>(b0 + c0) * K + (t - 1)) * Ds + q0 * 8;
+          const size_t seq_stride = static_cast<size_t>(K) * Ds;
+          auto at = [&](int bb, int cq) { return reinterpret_cast<const uint32_t*>(src + bb * seq_stride + cq * 8); };
+          for (int bb = bb0, cq = cq0; bb < nb && got;) {
+            // a batch: item (bb, cq) of this lane and the kPollBatch - 1 after it; every load is issued
+            // before any is checked
+            const int bs = bb, cs = cq;
             uint4 v[kPollBatch];
 #pragma unroll
-            for (int i = 0; i < kPollBatch; ++i) {  // issue every load first, then check
-              const int e = e0 + i * 32;
-              if (e < total) {
-                const size_t m = static_cast<size_t>(b0 + c0 + e / ncq) * K + (t - 1);
-                v[i] = ld_relaxed_v4(reinterpret_cast<const uint32_t*>(hxp + m * Ds + (q0 + e % ncq) * 8));
+            for (int i = 0; i < kPollBatch; ++i) {
+              if (bb < nb) v[i] = ld_relaxed_v4(at(bb, cq));
+              advance(bb, cq);
+            }
+            // late ones: wait for the first, then read all that were late again, together (one after
+            // another, each a round trip, made steps of 4.2 us up to 10 at B = 32)
+            while (true) {
+              int lb = -1, lq = 0, b1 = bs, c1 = cs;
+#pragma unroll
+              for (int i = 0; i < kPollBatch; ++i) {
+                if (lb < 0 && b1 < nb && !all_written(v[i])) {
+                  lb = b1;
+                  lq = c1;
+                }
+                advance(b1, c1);
+              }
+              if (lb < 0) break;
+              uint4 x;
+              got = poll_packed(at(lb, lq), x);
+              if (!got) break;
+              b1 = bs;
+              c1 = cs;
+#pragma unroll
+              for (int i = 0; i < kPollBatch; ++i) {
+                if (b1 < nb && !all_written(v[i])) v[i] = ld_relaxed_v4(at(b1, c1));
+                advance(b1, c1);
               }
             }
+            int b1 = bs, c1 = cs;
 #pragma unroll
             for (int i = 0; i < kPollBatch; ++i) {
-              const int e = e0 + i * 32;
-              if (e < total && got) {
-                const int bb = e / ncq, cq = q0 + e % ncq;
-                if (!all_written(v[i])) {
-                  const size_t m = static_cast<size_t>(b0 + c0 + bb) * K + (t - 1);
-                  got = poll_packed(hxp + m * Ds + cq * 8, v[i]);
-                  // the batch was early: by now its other late states are probably there, so they are
-                  // read again together rather than one round trip after another (B = 32: steps of 4.2 to
-                  // 10 us became 4.2; batches of 16 lose to it: 6.0 against 6.35 at B = 64)
-#pragma unroll
-                  for (int i2 = kPairs == 1 ? i + 1 : kPollBatch; i2 < kPollBatch; ++i2) {
-                    const int e2 = e0 + i2 * 32;
-                    if (e2 < total && !all_written(v[i2])) {
-                      const size_t m2 = static_cast<size_t>(b0 + c0 + e2 / ncq) * K + (t - 1);
-                      v[i2] = ld_relaxed_v4(reinterpret_cast<const uint32_t*>(hxp + m2 * Ds + (q0 + e2 % ncq) * 8));
-                    }
-                  }
-                }
-                *reinterpret_cast<uint4*>(hsm + static_cast<size_t>(bb) * ldw + cq * 8) =
+              if (b1 < nb && got)
+                *reinterpret_cast<uint4*>(hsm + static_cast<size_t>(b1) * ldw + (q0 + c1) * 8) =
                     make_uint4(unpack_states(v[i].x), unpack_states(v[i].y), unpack_states(v[i].z), unpack_states(v[i].w));
-              }
+              advance(b1, c1);
             }
           }
         } else {
@@ -795,7 +820,7 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
           float sum = 0.f;
 #pragma unroll
           for (int ww = 0; ww < kGruWarps; ++ww) sum += red[(static_cast<size_t>(ww) * tiles + tile) * 128 + w];
-          const int mt = tile / nt_count, nt = tile % nt_count;
+          const int mt = tile >= 2 * nt_count ? 2 : tile >= nt_count ? 1 : 0, nt = tile - mt * nt_count;  // kMaxMt is 3
           gsm[static_cast<size_t>(mt * 16 + w / 8) * gsm_ld + nt * 8 + (w % 8)] = sum;
         }
         __syncthreads();
@@ -805,7 +830,7 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
       for (int rr = 0; rr < kPairs; ++rr) {
         const int e = tid + rr * kGruThreads;
         if (e >= nb * Uc) break;
-        const int bb = e / Uc, jl = e % Uc;
+        const int bb = pb[rr], jl = pj[rr];
         const int j = j0 + jl;
         const int bl = c0 + bb;  // sequence index within this CTA
         const size_t m = static_cast<size_t>(b0 + bl) * K + t;
