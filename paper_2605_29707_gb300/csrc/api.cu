@@ -192,15 +192,19 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
   // tile above the average (V = 151936, 152 CTAs: eight tiles against 7.81), and the launch takes as
   // long as its longest chunk; so the chunks are made equal to within the operand's eight rows and
   // the last tile of each is shorter (B = 1, H = 4096: 217.8 -> 214.3 us a step; B = 2 225.8 -> 220.5).
-  p.w_per_chunk = ceil_div(p.w_tiles, per_tok);
-  p.rows_chunk = p.w_per_chunk * (p.swap ? 128 : p.bn);
-  if (even_chunks && p.swap && p.w_per_chunk > 1) {
-    p.rows_chunk = ceil_div(ceil_div(V, per_tok), 8) * 8;
-    p.w_per_chunk = ceil_div(p.rows_chunk, 128);
-  }
-  p.tail_rows = p.rows_chunk - (p.w_per_chunk - 1) * (p.swap ? 128 : p.bn);
-  p.nchunks = ceil_div(V, p.rows_chunk);
-  p.grid = p.tok_tiles * p.nchunks;
+  auto split = [&](bool even) {
+    const int tile = p.swap ? 128 : p.bn;
+    p.w_per_chunk = ceil_div(p.w_tiles, per_tok);
+    p.rows_chunk = p.w_per_chunk * tile;
+    if (even && p.swap && p.w_per_chunk > 1) {
+      p.rows_chunk = ceil_div(ceil_div(V, per_tok), 8) * 8;
+      p.w_per_chunk = ceil_div(p.rows_chunk, tile);
+    }
+    p.tail_rows = p.rows_chunk - (p.w_per_chunk - 1) * tile;
+    p.nchunks = ceil_div(V, p.rows_chunk);
+    p.grid = p.tok_tiles * p.nchunks;
+  };
+  split(even_chunks);
 
   if (head) {
     p.u_in_gru = p.swap;
@@ -221,9 +225,9 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     // that the first whole tiles do not wait for an epilogue), so a larger D costs only TMEM
     // columns and a later epilogue; a short estimate, or too few blocks (4 at BN = 128), costs a
     // wait at the checkpoint, never correctness.
+    const double t_gru_us = 12.0 + K * (4.5 + 0.5 * B);
     {
       const double t_seg1_us = 128.0 * H * 2.0 * p.grid / 6.6e6;
-      const double t_gru_us = 12.0 + K * (4.5 + 0.5 * B);
       int d = static_cast<int>(std::ceil(t_gru_us / t_seg1_us)) + 1;
       int dmax = p.w_per_chunk < 512 / p.bn ? p.w_per_chunk : 512 / p.bn;
       if (p.bn <= 32 && 512 / p.bn - 2 < dmax) dmax = 512 / p.bn - 2;
@@ -233,6 +237,9 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
       p.deep = d < p.w_per_chunk && deep_smem > 0 && static_cast<size_t>(deep_smem) + p.gru.smem + 2560 <= 228 * 1024;
     }
     p.overlap = p.u_in_gru && vsm > 0 && static_cast<size_t>(vsm) + p.gru.smem + 2048 <= 228 * 1024;
+    // Where the GRU outlasts the whole stream, whole tiles on fewer CTAs leave it more of the chip (B = 2,
+    // K = 8, V = 41511: 98.4 us on 109 CTAs against 101.8 on 149).
+    if (p.overlap && t_gru_us > p.w_per_chunk * 128.0 * H * 2.0 * p.grid / 6.6e6) split(false);
     // With the overlap, chain the whole head: the gather, both projection GEMMs and the GRU
     // each let the next kernel launch early, so that the GRU's CTAs (and with them the
     // vocabulary stream) start while the projections still run.
