@@ -94,7 +94,6 @@ struct Plan {
   bool u_in_gru;  // small M: u finished inside the GRU kernel; large M: W1 GEMM + finalize
   bool overlap;   // vocab GEMM launched as a programmatic dependent of the GRU (deferred W2)
   int defer_tiles;  // leading tiles per CTA whose W2 segment waits for the GRU
-  bool deep;      // overlap: the vocab GEMM's ring is one stage deeper
   int tmem_cols;  // TMEM columns of the vocab GEMM
   // workspace layout (offsets in bytes)
   size_t ctrl_bytes, clear_bytes;  // clear_bytes from off_ctrl: the control words (+ hx, fused)
@@ -216,7 +215,7 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     // Overlap the GRU with the W_lm stream when a deferred-mode vocab CTA and a GRU CTA fit on
     // one SM (228 KB of shared memory, 1 KB reserved per CTA) and every tile of a CTA can keep
     // its own TMEM accumulator until u is ready.
-    const int vsm = dm::tc_softmax_deferred_smem(p.bn, false);
+    const int vsm = dm::tc_softmax_deferred_smem(p.bn, p.kmax);
     // The first D tiles of each CTA wait for u; the rest run whole.  Pass 0 streams only the
     // W_lm segment of those D tiles (128 x H bf16 per CTA and tile, about 6.6 TB/s over the
     // grid), so D covers the GRU's expected time (12 us + K steps of 4.5 + 0.5 B us, generous
@@ -232,9 +231,6 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
       int dmax = p.w_per_chunk < 512 / p.bn ? p.w_per_chunk : 512 / p.bn;
       if (p.bn <= 32 && 512 / p.bn - 2 < dmax) dmax = 512 / p.bn - 2;
       p.defer_tiles = d < 1 ? 1 : (d > dmax ? dmax : d);
-      // a deeper ring where the stream outlasts the GRU (see launch_tc_softmax_deferred)
-      const int deep_smem = dm::tc_softmax_deferred_smem(p.bn, true);
-      p.deep = d < p.w_per_chunk && deep_smem > 0 && static_cast<size_t>(deep_smem) + p.gru.smem + 2560 <= 228 * 1024;
     }
     p.overlap = p.u_in_gru && vsm > 0 && static_cast<size_t>(vsm) + p.gru.smem + 2048 <= 228 * 1024;
     // Where the GRU outlasts the whole stream, whole tiles on fewer CTAs leave it more of the chip (B = 2,
@@ -633,7 +629,7 @@ int run_step_launches(const Plan& P, const void* hidden, const int32_t* ids, con
     if (P.head && !P.u_in_gru && P.pair) tp.pdl_wait = 3;
     ts = timing_open(DOMINO_KERNEL_VOCAB, st);
     if (P.overlap)
-      rc = cuda_rc(dm::launch_tc_softmax_deferred(P.bn, P.kmax, P.deep, maps, tp, P.grid, st));
+      rc = cuda_rc(dm::launch_tc_softmax_deferred(P.bn, P.kmax, maps, tp, P.grid, st));
     else
       rc = cuda_rc(dm::launch_tc_gemm(dm::kModeSoftmax, P.bn, P.swap, P.kmax, maps, tp, P.grid, st));
     timing_close(ts, st);

@@ -62,16 +62,16 @@ cudaError_t launch_tc_gemm(int mode, int bn, bool swap, int kmax, const CUtensor
 cudaError_t launch_tc_store_dependent(const CUtensorMap* maps, const TcParams& p, int grid, cudaStream_t stream);
 // Deferred-segment vocabulary GEMM launched as a programmatic dependent of the GRU kernel
 // (bn 16 to 128; fewer pipeline stages so that its CTAs fit beside the GRU's on one SM).
-// deep: a ring one stage deeper (bn 16 and 32).
-cudaError_t launch_tc_softmax_deferred(int bn, int kmax, bool deep, const CUtensorMap* maps, const TcParams& p,
-                                       int grid, cudaStream_t stream);
-// Shared memory one deferred-mode CTA uses (for the co-residency budget); 0: no such form.
-int tc_softmax_deferred_smem(int bn, bool deep);
-// The launches for 8-entry top-k lists (kmax = 8; tc_softmax_k8.cu).
+cudaError_t launch_tc_softmax_deferred(int bn, int kmax, const CUtensorMap* maps, const TcParams& p, int grid,
+                                       cudaStream_t stream);
+// Shared memory one deferred-mode CTA uses (for the co-residency budget).
+int tc_softmax_deferred_smem(int bn, int kmax);
+// The same three for 8-entry top-k lists (kmax = 8; tc_softmax_k8.cu).
 cudaError_t launch_tc_softmax_k8(int bn, bool swap, const CUtensorMap* maps, const TcParams& p, int grid,
                                  cudaStream_t stream);
-cudaError_t launch_tc_softmax_deferred_k8(int bn, bool deep, const CUtensorMap* maps, const TcParams& p, int grid,
+cudaError_t launch_tc_softmax_deferred_k8(int bn, const CUtensorMap* maps, const TcParams& p, int grid,
                                           cudaStream_t stream);
+int tc_softmax_deferred_smem_k8(int bn);
 // Tokens on M in CTA pairs (p.pair, bn 256): the 2-SM MMA variant (tc_pair.cuh); the
 // weight boxes are 128 rows high.
 cudaError_t launch_tc_vocab_pair(int kmax, const CUtensorMap* maps, const TcParams& p, int grid, cudaStream_t stream);

@@ -25,30 +25,27 @@ cudaError_t launch_tc_softmax(int bn, bool swap, int kmax, const CUtensorMap* ma
   return cudaErrorInvalidValue;
 }
 
-// Deferred variants: stages that leave a GRU CTA (78 KB) room on the same SM, 6 (7), 5 (6), 5 and 4 for
-// BN = 16, 32, 64 and 128 (118 to 150 KB).  The deeper rings of BN = 16 and 32 pay where the stream
-// bounds the step (H = 4096: B = 1 218.2 -> 214.8 us, B = 2 224.7 -> 220.2) and cost where the GRU
-// does, which they slow down (H = 2048, B = 2: 154.9 -> 160.0); see Plan::deep.
-cudaError_t launch_tc_softmax_deferred(int bn, int kmax, bool deep, const CUtensorMap* maps, const TcParams& p,
-                                       int grid, cudaStream_t s) {
+// Deferred variants: the stages that leave a GRU CTA (80 KB) room on the same SM -- 6, 5, 5 and 4 for
+// BN = 16, 32, 64 and 128 (118 to 150 KB).
+cudaError_t launch_tc_softmax_deferred(int bn, int kmax, const CUtensorMap* maps, const TcParams& p, int grid,
+                                       cudaStream_t s) {
   if (p.defer < 1 || p.defer > kMaxBlocks || p.defer * bn > p.tmem_cols) return cudaErrorInvalidValue;
-  if (kmax == 8) return launch_tc_softmax_deferred_k8(bn, deep, maps, p, grid, s);
-#define DM_SD(BN, KM, ST, DEEP)              \
-  if (bn == BN && kmax == KM && deep == DEEP) \
-    return launch_tc_instance<BN, true, kModeSoftmax, KM, ST>(maps, p, grid, s, true);
-  DM_SD(16, 16, 6, false) DM_SD(16, 32, 6, false) DM_SD(32, 16, 5, false) DM_SD(32, 32, 5, false)
-  DM_SD(16, 16, 7, true) DM_SD(16, 32, 7, true) DM_SD(32, 16, 6, true) DM_SD(32, 32, 6, true)
-  DM_SD(64, 16, 5, false) DM_SD(64, 32, 5, false) DM_SD(128, 16, 4, false) DM_SD(128, 32, 4, false)
+  if (kmax == 8) return launch_tc_softmax_deferred_k8(bn, maps, p, grid, s);
+#define DM_SD(BN, KM, ST) \
+  if (bn == BN && kmax == KM) return launch_tc_instance<BN, true, kModeSoftmax, KM, ST>(maps, p, grid, s, true);
+  DM_SD(16, 16, 6) DM_SD(16, 32, 6) DM_SD(32, 16, 5) DM_SD(32, 32, 5)
+  DM_SD(64, 16, 5) DM_SD(64, 32, 5) DM_SD(128, 16, 4) DM_SD(128, 32, 4)
 #undef DM_SD
   return cudaErrorInvalidValue;
 }
 
-int tc_softmax_deferred_smem(int bn, bool deep) {
+int tc_softmax_deferred_smem(int bn, int kmax) {
+  if (kmax == 8) return tc_softmax_deferred_smem_k8(bn);
   // the list length takes no shared memory in this orientation
-  if (bn == 16) return deep ? TcCfg<16, true, kModeSoftmax, 8, 7>::kSmemBytes : TcCfg<16, true, kModeSoftmax, 8, 6>::kSmemBytes;
-  if (bn == 32) return deep ? TcCfg<32, true, kModeSoftmax, 8, 6>::kSmemBytes : TcCfg<32, true, kModeSoftmax, 8, 5>::kSmemBytes;
-  if (bn == 64 && !deep) return TcCfg<64, true, kModeSoftmax, 8, 5>::kSmemBytes;
-  if (bn == 128 && !deep) return TcCfg<128, true, kModeSoftmax, 8, 4>::kSmemBytes;
+  if (bn == 16) return TcCfg<16, true, kModeSoftmax, 16, 6>::kSmemBytes;
+  if (bn == 32) return TcCfg<32, true, kModeSoftmax, 16, 5>::kSmemBytes;
+  if (bn == 64) return TcCfg<64, true, kModeSoftmax, 16, 5>::kSmemBytes;
+  if (bn == 128) return TcCfg<128, true, kModeSoftmax, 16, 4>::kSmemBytes;
   return 0;
 }
 

@@ -17,17 +17,21 @@ cudaError_t launch_tc_softmax_k8(int bn, bool swap, const CUtensorMap* maps, con
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_tc_softmax_deferred_k8(int bn, bool deep, const CUtensorMap* maps, const TcParams& p, int grid,
+cudaError_t launch_tc_softmax_deferred_k8(int bn, const CUtensorMap* maps, const TcParams& p, int grid,
                                           cudaStream_t s) {
-  if (bn == 16)
-    return deep ? launch_tc_instance<16, true, kModeSoftmax, 8, 7>(maps, p, grid, s, true)
-                : launch_tc_instance<16, true, kModeSoftmax, 8, 6>(maps, p, grid, s, true);
-  if (bn == 32)
-    return deep ? launch_tc_instance<32, true, kModeSoftmax, 8, 6>(maps, p, grid, s, true)
-                : launch_tc_instance<32, true, kModeSoftmax, 8, 5>(maps, p, grid, s, true);
-  if (bn == 64 && !deep) return launch_tc_instance<64, true, kModeSoftmax, 8, 5>(maps, p, grid, s, true);
-  if (bn == 128 && !deep) return launch_tc_instance<128, true, kModeSoftmax, 8, 4>(maps, p, grid, s, true);
+  if (bn == 16) return launch_tc_instance<16, true, kModeSoftmax, 8, 6>(maps, p, grid, s, true);
+  if (bn == 32) return launch_tc_instance<32, true, kModeSoftmax, 8, 5>(maps, p, grid, s, true);
+  if (bn == 64) return launch_tc_instance<64, true, kModeSoftmax, 8, 5>(maps, p, grid, s, true);
+  if (bn == 128) return launch_tc_instance<128, true, kModeSoftmax, 8, 4>(maps, p, grid, s, true);
   return cudaErrorInvalidValue;
+}
+
+int tc_softmax_deferred_smem_k8(int bn) {
+  if (bn == 16) return TcCfg<16, true, kModeSoftmax, 8, 6>::kSmemBytes;
+  if (bn == 32) return TcCfg<32, true, kModeSoftmax, 8, 5>::kSmemBytes;
+  if (bn == 64) return TcCfg<64, true, kModeSoftmax, 8, 5>::kSmemBytes;
+  if (bn == 128) return TcCfg<128, true, kModeSoftmax, 8, 4>::kSmemBytes;
+  return 0;
 }
 
 }  // namespace dm
