@@ -270,8 +270,8 @@ DOMINO_API int domino_verify_tree_sample(const float* target_logits, const int32
  *   per SM; a CTA's shared memory (at most 225 KB) holds u of every sequence (4 B r) and its
  *   share of the base logits (4 B ceil(V / SMs) rows), plus, for r <= 256, as many of its W2
  *   rows as fit (its first 512 W2 rows live in the tensor memory, all of it, of the SM for the
- *   whole call; with the input table, B <= 2 and r a multiple of 64, 128-row W2 blocks in tensor
- *   and shared memory instead, for the tensor cores), or,
+ *   whole call; with r a multiple of 64, 128-row W2 blocks in tensor and shared memory instead, for
+ *   the tensor cores, except for domino_rollout_sample at B > 2 or without the input table), or,
  *   for r > 256, a 96 KB ring W2 streams through every step (those shares rounded up to whole
  *   ring chunks).  Sizes whose u and base-logit share alone exceed 225 KB return
  *   DOMINO_ERR_INVALID_ARG.

@@ -10,7 +10,9 @@
 //   tree     merge the partials -> lse, top-k log-probs; best-first draft tree
 // Other batches: memset (the control words: status, merge counters), gather (id check, state
 // words cleared; E = emb[ids] unless a table is given), tc store Xp = E . W_ih^T (not with a
-// table), tc store Up = hidden . W1[:, :H]^T, gru, tc soft, tree; large M moves the W1 GEMM
+// table), tc store Up = hidden . W1[:, :H]^T, gru, tc soft, tree; up to 128 positions each is a
+// programmatic dependent of the one before it and the W_lm segment streams beside the GRU, as
+// above, on 64- and 128-column accumulator blocks that are used in turn; large M moves the W1 GEMM
 // (both halves) and a SiLU kernel (u_finalize) after the GRU, and launches X, GRU, W1,
 // u_finalize and the vocabulary GEMM on CTA pairs each as a programmatic dependent of the kernel
 // before it (the pair kernel waits for u only before its W2 segment).  With the correction
@@ -191,6 +193,7 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
   // tile above the average (V = 151936, 152 CTAs: eight tiles against 7.81), and the launch takes as
   // long as its longest chunk; so the chunks are made equal to within the operand's eight rows and
   // the last tile of each is shorter (B = 1, H = 4096: 217.8 -> 214.3 us a step; B = 2 225.8 -> 220.5).
+  // Not where the GRU outlasts the stream (below).
   auto split = [&](bool even) {
     const int tile = p.swap ? 128 : p.bn;
     p.w_per_chunk = ceil_div(p.w_tiles, per_tok);

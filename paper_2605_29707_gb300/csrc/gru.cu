@@ -4,10 +4,12 @@
 // The recurrence is the only sequential part of the step: K dependent steps, each needing the
 // full previous state of a sequence.  One cooperative launch keeps the W_hh rows of a block of
 // hidden units resident in shared memory for all K steps and computes W_hh . h_{t-1} on the
-// tensor cores (mma.sync, bf16 operands, fp32 accumulation).  States cross CTAs through L2 as
-// tagged words (bf16 value in the high half, the step's 16-bit tag in the low half; one row per
-// (sequence, position)), so a CTA waits for exactly the data it reads: no grid barrier and no
-// release fence.  Every wait is bounded.
+// tensor cores (mma.sync, bf16 operands, fp32 accumulation).  States cross CTAs through L2, one row
+// per (sequence, position), in a form that shows whether a value is written: as tagged words (bf16
+// value in the high half, the step's 16-bit tag in the low half) beside the vocabulary stream, as
+// packed 16-bit values in launches that share no SM with it.  A CTA so waits for exactly the data
+// it reads: no grid barrier and no release fence.  Every wait is bounded.  A step (about 4 us at
+// H = 4096, B = 32) is bound by that exchange, not by its MMAs.
 #include <math.h>
 
 #include <atomic>

@@ -88,7 +88,7 @@ struct GatherParams {
   const int32_t* ids;       // [M]
   const __nv_bfloat16* emb; // [V, H]
   __nv_bfloat16* E;         // [M, H] or nullptr (validate only)
-  uint32_t* hx;             // [M, Ds] tagged GRU states to clear, or nullptr
+  uint32_t* hx;             // [M, Ds] GRU state words to clear, or nullptr
   int M, H, V, Ds;
   int* status;
 };

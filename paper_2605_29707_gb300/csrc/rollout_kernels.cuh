@@ -22,10 +22,18 @@
 // Every wait is bounded.
 //
 // W2 (V x r bf16, 78 MB at the Qwen3 vocabulary) is the operand phase C reads every step.  With
-// r <= 256 the resident kernel keeps each CTA's slice of it on chip for the whole block: 512
+// r <= 256 the resident kernel keeps each CTA's slice of it on chip for the whole block.  With r a
+// multiple of 64 phase C runs on the tensor cores (kMma): 128-row blocks of W2 as the A operand in
+// tensor memory and in shared memory, u_j as the B operand in three bf16 terms (exact), the rows
+// past the blocks read through L2 as 16-row mma.sync tiles.  Otherwise, and for the inverse-CDF
+// rule at B > 2 or without the table (its draw is decided by the order of the fp32 sums): 512
 // rows in the SM's tensor memory (used as storage: written once with tcgen05.st, read with
-// tcgen05.ld), as many rows as fit in shared memory, and the few rows left read through L2.
+// tcgen05.ld), as many rows as fit in shared memory, the rest through L2, on the CUDA cores.
 // Wider r uses the streamed kernel, which feeds W2 through a shared-memory ring every step.
+//
+// The steps with the table (kFast: h of every sequence in every CTA's shared memory) have one grid
+// barrier; without it, or where h does not fit, three phases.  The two are kernels of their own,
+// since each needs the whole register budget.
 #pragma once
 
 #include <math.h>

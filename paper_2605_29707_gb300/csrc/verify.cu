@@ -4,10 +4,10 @@
 // (temperature 0: the target's choice after a node is its argmax) and sampled (temperature T > 0:
 // its choice is a draw from softmax(logits / T) with the caller's uniform).
 //
-// Row argmax: a cluster of CTAs (kSplit, or two when the rows are many) per row of target logits (the target's next-token logits
-// after the anchor, row 0, and after each tree node i, row i + 1); each CTA finds the greatest
-// value of its slice of the row and, among equal values, the lowest id, and the cluster's first
-// CTA combines the slices through distributed shared memory.  Walk: one warp per sequence
+// Row argmax: a cluster of CTAs (kSplit, or two when the rows are many) per row of target logits
+// (the target's next-token logits after the anchor, row 0, and after each tree node i, row i + 1);
+// each CTA finds the greatest value of its slice of the row and, among equal values, the lowest
+// id, and the cluster's first CTA combines the slices through distributed shared memory.  Walk: one warp per sequence
 // starts at the anchor, takes the argmax of the current node's row and moves to the child
 // carrying that token (the lowest node index if several do), until no child does; that argmax
 // is the bonus token.
