@@ -188,17 +188,15 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
   if (per_tok < 1) per_tok = 1;
   // Tokens on M: pairs of CTAs with consecutive token tiles share each weight tile (2-SM MMA).
   p.pair = !p.swap && p.tok_tiles % 2 == 0;
-  // Each CTA streams a contiguous chunk of the vocabulary in tiles of 128 (256) rows.  Up to 128
-  // positions, where the launch is bound by HBM, whole tiles would leave the longest chunk up to one
-  // tile above the average (V = 151936, 152 CTAs: eight tiles against 7.81), and the launch takes as
-  // long as its longest chunk; so the chunks are made equal to within the operand's eight rows and
-  // the last tile of each is shorter (B = 1, H = 4096: 217.8 -> 214.3 us a step; B = 2 225.8 -> 220.5).
-  // Not where the GRU outlasts the stream (below).
+  // Each CTA streams a contiguous chunk of the vocabulary in tiles of 128 (256) rows.  Whole tiles
+  // leave the longest chunk up to one tile above the average; equal chunks (to within the operand's
+  // eight rows, the last tile of each shorter) even that out over all the CTAs.  They are taken for 33
+  // to 128 positions beside the GRU (below).
   auto split = [&](bool even) {
     const int tile = p.swap ? 128 : p.bn;
     p.w_per_chunk = ceil_div(p.w_tiles, per_tok);
     p.rows_chunk = p.w_per_chunk * tile;
-    if (even && p.swap && p.w_per_chunk > 1) {
+    if (even && p.w_per_chunk > 1) {
       p.rows_chunk = ceil_div(ceil_div(V, per_tok), 8) * 8;
       p.w_per_chunk = ceil_div(p.rows_chunk, tile);
     }
@@ -206,7 +204,7 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     p.nchunks = ceil_div(V, p.rows_chunk);
     p.grid = p.tok_tiles * p.nchunks;
   };
-  split(even_chunks);
+  split(false);
 
   if (head) {
     p.u_in_gru = p.swap;
@@ -219,6 +217,14 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     // one SM (228 KB of shared memory, 1 KB reserved per CTA) and every tile of a CTA can keep
     // its own TMEM accumulator until u is ready.
     const int vsm = dm::tc_softmax_deferred_smem(p.bn, p.kmax);
+    p.overlap = p.u_in_gru && vsm > 0 && static_cast<size_t>(vsm) + p.gru.smem + 2048 <= 228 * 1024;
+    // Equal chunks on the wide accumulator blocks, whose tiles' epilogues count (us, whole against
+    // equal: B = 6, V = 60000 231.1 -> 222.6; B = 8, V = 100000 275.1 -> 270.4; B = 4, V = 41511 163.1 -> 158.6).
+    // On 16 and 32 columns the stream alone counts, fewer CTAs carry it as well, and the SMs
+    // without one speed the GRU up: whole tiles (equal against whole: B = 1, V = 151936 219.7 -> 216.2,
+    // V = 60000 139.2 -> 132.4; B = 2, V = 100000 192.5 -> 183.7; only B = 2, V = 130000 202.6 -> 210.1
+    // is the other way).  Without the head whole tiles too (B = 4, V = 41511 88.7 -> 84.2).
+    if (even_chunks && p.overlap && p.bn >= 64) split(true);
     // The first D tiles of each CTA wait for u; the rest run whole.  Pass 0 streams only the
     // W_lm segment of those D tiles (128 x H bf16 per CTA and tile, about 6.6 TB/s over the
     // grid), so D covers the GRU's expected time (12 us + K steps of 4.5 + 0.5 B us, generous
@@ -227,18 +233,14 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     // that the first whole tiles do not wait for an epilogue), so a larger D costs only TMEM
     // columns and a later epilogue; a short estimate, or too few blocks (4 at BN = 128), costs a
     // wait at the checkpoint, never correctness.
-    const double t_gru_us = 12.0 + K * (4.5 + 0.5 * B);
     {
       const double t_seg1_us = 128.0 * H * 2.0 * p.grid / 6.6e6;
+      const double t_gru_us = 12.0 + K * (4.5 + 0.5 * B);
       int d = static_cast<int>(std::ceil(t_gru_us / t_seg1_us)) + 1;
       int dmax = p.w_per_chunk < 512 / p.bn ? p.w_per_chunk : 512 / p.bn;
       if (p.bn <= 32 && 512 / p.bn - 2 < dmax) dmax = 512 / p.bn - 2;
       p.defer_tiles = d < 1 ? 1 : (d > dmax ? dmax : d);
     }
-    p.overlap = p.u_in_gru && vsm > 0 && static_cast<size_t>(vsm) + p.gru.smem + 2048 <= 228 * 1024;
-    // Where the GRU outlasts the whole stream, whole tiles on fewer CTAs leave it more of the chip (B = 2,
-    // K = 8, V = 41511: 98.4 us on 109 CTAs against 101.8 on 149).
-    if (p.overlap && t_gru_us > p.w_per_chunk * 128.0 * H * 2.0 * p.grid / 6.6e6) split(false);
     // With the overlap, chain the whole head: the gather, both projection GEMMs and the GRU
     // each let the next kernel launch early, so that the GRU's CTAs (and with them the
     // vocabulary stream) start while the projections still run.

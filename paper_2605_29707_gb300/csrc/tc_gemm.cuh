@@ -31,6 +31,7 @@ struct TcCfg {
   static constexpr int kBBytes = BN * 128;   // BN rows x 64 bf16
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kTPT = SWAP ? 128 / BN : 1;  // epilogue threads per token (swap)
+  static constexpr bool kEven = MODE == kModeSoftmax && SWAP && BN >= 64;  // see tc_get_item
   // Vocabulary rows transposed at a time: what gives each epilogue thread one chunk of 32 values
   // (16 for BN = 16).  A whole 128-row tile at BN = 64 and 128 would take 33 and 66 KB of shared
   // memory instead of 17, which the ring needs (and, in the deferred variants, the GRU's CTA).
@@ -63,10 +64,10 @@ struct TcItem {
   bool tail;       // softmax mode with swap: the chunk's last tile
 };
 
-// TILE: weight rows of a tile.  EVEN: equal chunks, whose last tile is shorter (weights
-// on the 128-row operand; with weights on N the launch is bound by the tensor cores, where equal
-// chunks gained under 1 % and the code for them cost up to 6 %; the loop's store-mode GEMM over the
-// vocabulary, whose CTAs take its tiles in turn, lost 2 % to them at B = 4).
+// TILE: weight rows of a tile.  EVEN: the plan may make equal chunks, whose last tile is shorter
+// (33 to 128 positions, see the split in api.cu; with weights on N the launch is bound by the tensor cores, where
+// equal chunks gained under 1 % and the code for them cost up to 6 %; the loop's store-mode GEMM over
+// the vocabulary, whose CTAs take its tiles in turn, lost 2 % to them at B = 4).
 template <int MODE, int TILE, bool EVEN>
 __device__ __forceinline__ bool tc_get_item(const TcParams& p, int i, TcItem& it) {
   const int nkb = p.nkb1 + p.nkb2;
@@ -83,6 +84,9 @@ __device__ __forceinline__ bool tc_get_item(const TcParams& p, int i, TcItem& it
       const int w = chunk * p.w_per_chunk + i;
       if (chunk >= p.nchunks || i >= p.w_per_chunk || w >= p.w_tiles) return false;
       it.w = w;
+      it.row0 = w * TILE;
+      it.rows = TILE;
+      it.tail = false;
     }
     return true;
   } else {
@@ -311,7 +315,7 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
       tma_prefetch_desc(&tmA2);
       tma_prefetch_desc(&tmB2);
     }
-    if (MODE == kModeSoftmax && SWAP) {
+    if (C::kEven) {
       tma_prefetch_desc(&tmT1);
       if (p.nkb2 > 0) tma_prefetch_desc(&tmT2);
     }
@@ -352,13 +356,13 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
       const int passes = p.defer ? 3 : 1;
       for (int pass = 0; pass < passes && ok; ++pass) {
       if (pass == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
-      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE, kTile, SWAP>(p, i, it); ++i) {
+      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE, kTile, C::kEven>(p, i, it); ++i) {
         if (pass < 2 && p.defer && i >= p.defer) break;
         const int kb_lo = (p.defer && pass == 1) ? p.nkb1 : it.kb0;
         const int kb_hi = (p.defer && pass == 0) ? p.nkb1 : it.kb1;
         for (int kb = kb_lo; kb < kb_hi; ++kb) {
           if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
-          const bool tail = MODE == kModeSoftmax && SWAP && it.tail;  // fewer weight rows, by their own maps
+          const bool tail = C::kEven && it.tail;  // fewer weight rows, by their own maps
           mbar_arrive_expect_tx(&full[stage], tail ? C::kBBytes + it.rows * 128 : C::kStageBytes);
           const bool seg2 = kb >= p.nkb1;
           const int kx = (seg2 ? kb - p.nkb1 : kb) * 64;
@@ -398,7 +402,7 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
       TcItem it;
       const int passes = p.defer ? 3 : 1;
       for (int pass = 0; pass < passes && ok; ++pass) {
-      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE, kTile, SWAP>(p, i, it); ++i) {
+      for (int i = (pass == 2 ? p.defer : 0); ok && tc_get_item<MODE, kTile, C::kEven>(p, i, it); ++i) {
         if (pass < 2 && p.defer && i >= p.defer) break;
         // a deferred tile (i < p.defer <= blocks) is its block's first; a block used before waits
         // for the epilogue of the tile it held
@@ -441,7 +445,7 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
     bool aborted = false;
     TcItem it;
     it.tok = 0;
-    for (int i = 0; tc_get_item<MODE, kTile, SWAP>(p, i, it); ++i) {
+    for (int i = 0; tc_get_item<MODE, kTile, C::kEven>(p, i, it); ++i) {
       const int nblk = tc_blocks<BN>(p), ab = i & (nblk - 1);
       const bool ok = mbar_wait(&tfull[ab], (i / nblk) & 1, abort_flag, p.status);
       if (epi_any(!ok)) { aborted = true; break; }
