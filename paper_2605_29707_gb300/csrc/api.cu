@@ -223,8 +223,10 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     // On 16 and 32 columns the stream alone counts, fewer CTAs carry it as well, and the SMs
     // without one speed the GRU up: whole tiles (equal against whole: B = 1, V = 151936 219.7 -> 216.2,
     // V = 60000 139.2 -> 132.4; B = 2, V = 100000 192.5 -> 183.7; only B = 2, V = 130000 202.6 -> 210.1
-    // is the other way).  Without the head whole tiles too (B = 4, V = 41511 88.7 -> 84.2).
-    if (even_chunks && p.overlap && p.bn >= 64) split(true);
+    // is the other way).  Without the head whole tiles too (B = 4, V = 41511 88.7 -> 84.2), and on 64
+    // columns where whole tiles keep nine tenths of the CTAs busy (B = 4, V = 151936 256.3 -> 252.3; at 128
+    // columns, B = 7, equal chunks take 307.2 against 307.9).
+    if (even_chunks && p.overlap && (p.bn == 128 || (p.bn == 64 && 10 * p.nchunks < 9 * per_tok))) split(true);
     // The first D tiles of each CTA wait for u; the rest run whole.  Pass 0 streams only the
     // W_lm segment of those D tiles (128 x H bf16 per CTA and tile, about 6.6 TB/s over the
     // grid), so D covers the GRU's expected time (12 us + K steps of 4.5 + 0.5 B us, generous

@@ -13,7 +13,8 @@ from tests.test_gpu_parity import _check, _run_gpu
 pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, 5, 152 * 136 - 3, 6), (2, 9, 152 * 248 + 1 - 152 * 8, 12), (3, 11, 152 * 136 - 3, 6),
-          (4, 16, 152 * 248 + 1 - 152 * 8, 12), (5, 13, 152 * 256, 8), (8, 16, 152 * 264 - 700, 8)]
+          (4, 16, 152 * 248 + 1 - 152 * 8, 12), (5, 13, 152 * 256, 8),
+          (5, 13, 152 * 248 + 1 - 152 * 8, 12), (8, 16, 152 * 264 - 700, 8)]
 
 
 @pytest.mark.parametrize("B,K,V,k", SHAPES)
