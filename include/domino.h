@@ -182,12 +182,22 @@ DOMINO_API int domino_check_status(const void* workspace, void* stream);
  *                              that a small-batch step (B <= 2 at K = 16) runs when the workspace
  *                              last held another kind or shape of step (or is fresh); `step` is
  *                              ignored, and a step that needs no clear withholds nothing;
+ *   DOMINO_HOLD_ROW_COPY       the next domino_verify_tree_sample launch does not copy part of row
+ *                              gru_cta (counted over all sequences) into shared memory; its wait
+ *                              for the copy runs out, the row is read directly instead, and the
+ *                              outputs are those of any other call; rows that are not copied so
+ *                              (V not a multiple of 4) withhold nothing;
  *   DOMINO_HOLD_OFF            disarms the hook.
  * The held CTA disarms the hook when its launch ends, so it affects one step.  Every kernel of
  * the held step still completes (its outputs are undefined) and the workspace stays usable: the
  * next step runs normally.  Synchronous (a copy to a device symbol); not for use while steps
  * run on other threads.  Returns DOMINO_OK, DOMINO_ERR_INVALID_ARG or DOMINO_ERR_CUDA. */
-enum domino_hold { DOMINO_HOLD_OFF = 0, DOMINO_HOLD_STATE = 1, DOMINO_HOLD_CLEAR_BARRIER = 2 };
+enum domino_hold {
+  DOMINO_HOLD_OFF = 0,
+  DOMINO_HOLD_STATE = 1,
+  DOMINO_HOLD_CLEAR_BARRIER = 2,
+  DOMINO_HOLD_ROW_COPY = 3
+};
 DOMINO_API int domino_debug_hold(int what, int gru_cta, int step);
 
 /* Static, human-readable name of a status code. */

@@ -35,6 +35,7 @@ DOMINO_STATIC_SCRATCH_BYTES = 16 << 20
 DOMINO_HOLD_OFF = 0
 DOMINO_HOLD_STATE = 1
 DOMINO_HOLD_CLEAR_BARRIER = 2
+DOMINO_HOLD_ROW_COPY = 3
 
 KERNEL_KINDS = ("gather", "gru_input_proj", "w1_hidden_proj", "gru", "vocab_gemm_softmax_topk", "merge_tree",
                 "rollout_base_gemm", "rollout_steps", "tree_verify")
@@ -277,5 +278,6 @@ def domino_rollout_sample_gumbel(hidden, anchors, seed, w_lm, head, B, K, H, V, 
 def domino_debug_hold(what, gru_cta=-1, step=-1) -> int:
     """Test hook: the next GRU launch's CTA ``gru_cta`` withholds its states of position ``step``
     (DOMINO_HOLD_STATE) or its clear-barrier arrival (DOMINO_HOLD_CLEAR_BARRIER); DOMINO_HOLD_OFF
-    disarms.  The step then reports DOMINO_ERR_TIMEOUT through its device status."""
+    disarms.  The step then reports DOMINO_ERR_TIMEOUT through its device status.
+    DOMINO_HOLD_ROW_COPY: the next sampled verification does not stage part of row ``gru_cta``."""
     return int(load().domino_debug_hold(int(what), int(gru_cta), int(step)))

@@ -845,7 +845,15 @@ const char* domino_status_string(int status) {
 int domino_abi_version(void) { return DOMINO_ABI_VERSION; }
 
 int domino_debug_hold(int what, int gru_cta, int step) {
-  if (what == DOMINO_HOLD_OFF) return cuda_rc(dm::arm_gru_hold(dm::kHoldOff, -1, -1));
+  if (what == DOMINO_HOLD_OFF) {
+    dm::arm_row_hold(-1);
+    return cuda_rc(dm::arm_gru_hold(dm::kHoldOff, -1, -1));
+  }
+  if (what == DOMINO_HOLD_ROW_COPY) {  // gru_cta: the row
+    if (gru_cta < 0) return DOMINO_ERR_INVALID_ARG;
+    dm::arm_row_hold(gru_cta);
+    return DOMINO_OK;
+  }
   if (what != DOMINO_HOLD_STATE && what != DOMINO_HOLD_CLEAR_BARRIER) return DOMINO_ERR_INVALID_ARG;
   if (gru_cta < 0 || (what == DOMINO_HOLD_STATE && (step < 0 || step >= kMaxK))) return DOMINO_ERR_INVALID_ARG;
   const int kind = what == DOMINO_HOLD_STATE ? dm::kHoldPublish : dm::kHoldClearBarrier;

@@ -247,6 +247,8 @@ cudaError_t launch_verify_greedy(const float* logits, const int32_t* parent, con
 // Row draws from softmax(logits / T) (inv_t = 1 / T) with one uniform per row, then the same walk;
 // a row slice of at most kMaxSampleSlice floats is staged in shared memory (V <= 8 of them).
 constexpr int kMaxSampleSlice = 53248;
+// Test hook (domino_debug_hold): the next launch withholds one copy of row `row` (-1: disarmed).
+void arm_row_hold(int row);
 cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, const int32_t* token,
                                  const float* uniforms, int B, int N, int V, float inv_t, int32_t* row_sample,
                                  int32_t* nodes, int32_t* count, int32_t* bonus, cudaStream_t stream);

@@ -19,6 +19,8 @@
 // cumulative sum (in id order) passes it.  The walk is the greedy one on the draws.
 #include <math.h>
 
+#include <atomic>
+
 #include "kernels.h"
 #include "ptx.cuh"
 
@@ -206,7 +208,8 @@ __device__ __forceinline__ float ld_cluster_f32(const void* local, uint32_t rank
 // contiguous run, then thread order, then slice order), so the draw is deterministic.
 __global__ void __launch_bounds__(kSampleThreads) row_sample_kernel(const float* __restrict__ logits, int V,
                                                                     float inv_t, const float* __restrict__ uniforms,
-                                                                    int32_t* __restrict__ row_sample, int ahead) {
+                                                                    int32_t* __restrict__ row_sample, int ahead,
+                                                                    int held) {
   extern __shared__ __align__(16) float s_x[];  // this CTA's slice of the row
   __shared__ float s_red[kSampleThreads / 32];
   __shared__ int s_nz[kSampleThreads / 32];  // each warp's last thread of non-zero run sum (-1: none)
@@ -226,8 +229,13 @@ __global__ void __launch_bounds__(kSampleThreads) row_sample_kernel(const float*
   const int len = max(0, min(V, lo + slice) - lo);
   const float u_row = tid == 0 ? __ldg(uniforms + row) : 0.f;  // issued early, used after the sums
 
-  // ---- stage the slice (asynchronous bulk copies, all in flight at once), slice maximum
+  // ---- stage the slice (asynchronous bulk copies, all in flight at once), slice maximum.  The entry
+  //      points have no status word, so a copy that has not landed within the limit is no error: the
+  //      thread reads what it needs of that chunk itself (the same bytes, should the copy still land)
+  //      and waits for the copies once more before it leaves.  `held`: the test hook's row (-1: none),
+  //      whose first chunk is not copied.
   float mx = -INFINITY;
+  bool late = false;
   if ((V & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
     const int ch = (slice / kStageChunks + 3) & ~3;  // floats per chunk (whole 16-byte units)
     if (tid == 0) {
@@ -236,7 +244,7 @@ __global__ void __launch_bounds__(kSampleThreads) row_sample_kernel(const float*
       const uint64_t pol = l2_policy_evict_first();
       for (int c = 0; c < kStageChunks; ++c) {
         const int f0 = c * ch, n = min(len, f0 + ch) - f0;
-        if (n > 0) {
+        if (n > 0 && !(c == 0 && static_cast<int>(row) == held)) {
           mbar_arrive_expect_tx(&s_bar[c], static_cast<uint32_t>(n) * 4);
           bulk_load(s_x + f0, x + lo + f0, static_cast<uint32_t>(n) * 4, &s_bar[c], pol);
         }
@@ -246,14 +254,15 @@ __global__ void __launch_bounds__(kSampleThreads) row_sample_kernel(const float*
         l2_prefetch_bulk(x + static_cast<size_t>(ahead) * V + lo, static_cast<uint32_t>(len) * 4);
     }
     __syncthreads();
-    const float4* s4 = reinterpret_cast<const float4*>(s_x);
+    const float4* x4 = reinterpret_cast<const float4*>(x + lo);
+    float4* s4 = reinterpret_cast<float4*>(s_x);
     for (int c = 0; c < kStageChunks; ++c) {
       const int f0 = c * ch, f1 = min(len, f0 + ch);
       if (f0 >= f1) break;
       const long long t0 = clock64();
-      while (!mbar_try_wait(&s_bar[c], 0))
-        if (clock64() - t0 > kWaitCycles) break;
+      while (!late && !mbar_try_wait(&s_bar[c], 0)) late = clock64() - t0 > kWaitCycles;
       for (int q = f0 / 4 + tid; q < f1 / 4; q += kSampleThreads) {
+        if (late) s4[q] = __ldg(x4 + q);
         const float4 f = s4[q];
         mx = fmaxf(mx, fmaxf(fmaxf(f.x, f.y), fmaxf(f.z, f.w)));
       }
@@ -401,8 +410,20 @@ __global__ void __launch_bounds__(kSampleThreads) row_sample_kernel(const float*
       if (lane == 0) row_sample[row] = lo + (y >= 0 ? y : (lastnz >= 0 ? lastnz : min(q0, len - 1)));
     }
   }
+  if (late) {  // every copy of this CTA has landed before it leaves (bounded)
+    const int ch = (slice / kStageChunks + 3) & ~3;
+    const long long t0 = clock64();
+    for (int c = 0; c < kStageChunks && c * ch < len; ++c)
+      while (!mbar_try_wait(&s_bar[c], 0) && clock64() - t0 <= kWaitCycles) {
+      }
+  }
   cluster_wait();  // no CTA leaves while another may still read its slice sum
 }
+
+// Test hook state (domino_debug_hold): the row of the next sampled verification whose first chunk is
+// not copied; -1: none.
+static std::atomic<int> g_held_row{-1};
+void arm_row_hold(int row) { g_held_row = row; }
 
 cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, const int32_t* token,
                                  const float* uniforms, int B, int N, int V, float inv_t, int32_t* row_sample,
@@ -431,7 +452,8 @@ cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, con
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, row_sample_kernel, logits, V, inv_t, uniforms, row_sample, kAhead);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, row_sample_kernel, logits, V, inv_t, uniforms, row_sample, kAhead,
+                                     g_held_row.exchange(-1));
   if (e != cudaSuccess) return e;
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
