@@ -31,14 +31,18 @@ struct TcCfg {
   static constexpr int kBBytes = BN * 128;   // BN rows x 64 bf16
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kTPT = SWAP ? 128 / BN : 1;  // epilogue threads per token (swap)
-  static constexpr bool kEven = MODE == kModeSoftmax && SWAP && BN >= 64;  // see tc_get_item
-  // Vocabulary rows transposed at a time: what gives each epilogue thread one chunk of 32 values
-  // (16 for BN = 16).  A whole 128-row tile at BN = 64 and 128 would take 33 and 66 KB of shared
-  // memory instead of 17, which the ring needs (and, in the deferred variants, the GRU's CTA).
-  static constexpr int kTrRows = 32 * kTPT < 128 ? 32 * kTPT : 128;
+  static constexpr bool kDeferred = ST > 0;         // beside the GRU
+  static constexpr bool kEven = MODE == kModeSoftmax && SWAP && BN >= 64 && kDeferred;  // see tc_get_item
+  // Vocabulary rows transposed at a time.  A kernel with the SM to itself takes the whole tile, so that
+  // all four epilogue warps stage at once, and a larger shared-memory budget for it (33 and 66 KB at
+  // BN = 64 and 128).  Beside the GRU's CTA there is no room for that, and a pass has the rows that
+  // give each epilogue thread one chunk of 32 values (16 for BN = 16).  In passes, and with the code
+  // for equal chunks, the epilogue bounds a short main loop: 8 sequences without the head at
+  // V = 151936 took 168 us at H = 2048 so, 147 now (221 and 218 at H = 4096).
+  static constexpr int kTrRows = !kDeferred || 32 * kTPT > 128 ? 128 : 32 * kTPT;
   static constexpr int kTrStride = kTrRows + kTPT;  // conflict-free transpose pitch (floats)
   static constexpr int kTrBytes = (SWAP && MODE == kModeSoftmax) ? BN * kTrStride * 4 : 0;
-  static constexpr int kBudget = 200 * 1024;
+  static constexpr int kBudget = (!kDeferred && SWAP && MODE == kModeSoftmax ? 225 : 200) * 1024;
   static constexpr int kSt0 = (kBudget - kTrBytes) / kStageBytes;
   static constexpr int kStages = ST > 0 ? ST : (kSt0 > 8 ? 8 : kSt0);
   static constexpr int kTmemCols =
@@ -65,9 +69,9 @@ struct TcItem {
 };
 
 // TILE: weight rows of a tile.  EVEN: the plan may make equal chunks, whose last tile is shorter
-// (33 to 128 positions, see the split in api.cu; with weights on N the launch is bound by the tensor cores, where
-// equal chunks gained under 1 % and the code for them cost up to 6 %; the loop's store-mode GEMM over
-// the vocabulary, whose CTAs take its tiles in turn, lost 2 % to them at B = 4).
+// (33 to 128 positions beside the GRU, see the split in api.cu; with weights on N the launch is bound by
+// the tensor cores, where equal chunks gained under 1 % and the code for them cost up to 6 %; the loop's
+// store-mode GEMM over the vocabulary, whose CTAs take its tiles in turn, lost 2 % to them at B = 4).
 template <int MODE, int TILE, bool EVEN>
 __device__ __forceinline__ bool tc_get_item(const TcParams& p, int i, TcItem& it) {
   const int nkb = p.nkb1 + p.nkb2;
@@ -492,8 +496,8 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
         tc_fence_before();
         mbar_arrive(&tempty[ab]);
       } else if constexpr (SWAP) {
-        // vocabulary rows on TMEM lanes, tokens on columns: stage kTrRows rows at a time through
-        // shared memory so that each thread owns one token and a strided slice of the rows
+        // vocabulary rows on TMEM lanes, tokens on columns: staged through shared memory, kTrRows rows at
+        // a time, so that each thread owns one token and a strided slice of the rows
         const int vrow = 32 * q + lane;
         const int v = it.row0 + vrow;
         const int vend = min(p.rows_w, it.row0 + it.rows);
@@ -503,29 +507,47 @@ __global__ void __launch_bounds__(ST > 0 ? 256 : 192, ST > 0 ? 2 : 1)
         const int sub = ep % C::kTPT;
         const float* trow = tr + tt * C::kTrStride;
         constexpr int kSub = BN < 32 ? BN : 32;
+        auto stage_rows = [&](int h0) {
+#pragma unroll
+          for (int c0 = 0; c0 < BN; c0 += kSub) {
+            float r[kSub];
+            if constexpr (BN < 32) tc_ld_x16(tcol + c0, r); else tc_ld_x32(tcol + c0, r);
+            tc_wait_ld();
+#pragma unroll
+            for (int j = 0; j < kSub; ++j) tr[(c0 + j) * C::kTrStride + vrow - h0] = r[j] + bv;
+          }
+          tc_fence_before();
+          mbar_arrive(&tempty[ab]);
+        };
+        if constexpr (C::kTrRows == 128) {
+          stage_rows(0);
+          named_bar_sync(1, 128);
+          const int left = vend - it.row0 - sub;  // valid entries: sub + TPT * j < vend - row0
+          const int nvalid_all = left <= 0 ? 0 : (left + C::kTPT - 1) / C::kTPT;
 #pragma unroll 1
-        for (int h0 = 0; h0 < 128; h0 += C::kTrRows) {
-          if (vrow >= h0 && vrow < h0 + C::kTrRows) {  // whole warps: kTrRows is a multiple of 32
+          for (int j0 = 0; j0 < BN; j0 += kSub) {
+            float r[kSub];
+            const float* sx = trow + sub + C::kTPT * j0;
 #pragma unroll
-            for (int c0 = 0; c0 < BN; c0 += kSub) {
-              float r[kSub];
-              if constexpr (BN < 32) tc_ld_x16(tcol + c0, r); else tc_ld_x32(tcol + c0, r);
-              tc_wait_ld();
-#pragma unroll
-              for (int j = 0; j < kSub; ++j) tr[(c0 + j) * C::kTrStride + vrow - h0] = r[j] + bv;
-            }
-            tc_fence_before();
-            mbar_arrive(&tempty[ab]);
+            for (int j = 0; j < kSub; ++j) r[j] = sx[C::kTPT * j];
+            stream_chunk<kSub, KMAX>(r, sx, C::kTPT, it.row0 + sub + C::kTPT * j0, C::kTPT, nvalid_all - j0, st.mx,
+                                     st.se, st.tv, st.ti);
           }
           named_bar_sync(1, 128);
-          const int vbase = it.row0 + h0 + sub;
-          const int left = vend - vbase;  // valid entries: vbase + TPT * j < vend
-          const int nvalid = left <= 0 ? 0 : (left + C::kTPT - 1) / C::kTPT;
-          float r[kSub];
+        } else {
+#pragma unroll 1
+          for (int h0 = 0; h0 < 128; h0 += C::kTrRows) {
+            if (vrow >= h0 && vrow < h0 + C::kTrRows) stage_rows(h0);  // whole warps: kTrRows is a multiple of 32
+            named_bar_sync(1, 128);
+            const int vbase = it.row0 + h0 + sub;
+            const int left = vend - vbase;  // valid entries: vbase + TPT * j < vend
+            const int nvalid = left <= 0 ? 0 : (left + C::kTPT - 1) / C::kTPT;
+            float r[kSub];
 #pragma unroll
-          for (int j = 0; j < kSub; ++j) r[j] = trow[sub + C::kTPT * j];
-          stream_chunk<kSub, KMAX>(r, trow + sub, C::kTPT, vbase, C::kTPT, nvalid, st.mx, st.se, st.tv, st.ti);
-          named_bar_sync(1, 128);
+            for (int j = 0; j < kSub; ++j) r[j] = trow[sub + C::kTPT * j];
+            stream_chunk<kSub, KMAX>(r, trow + sub, C::kTPT, vbase, C::kTPT, nvalid, st.mx, st.se, st.tv, st.ti);
+            named_bar_sync(1, 128);
+          }
         }
       } else {
         // tokens on TMEM lanes: each thread streams its own row across the vocabulary tile
