@@ -538,27 +538,33 @@ __device__ __forceinline__ void bf4(const __nv_bfloat16* p, float (&f)[4]) {
 
 // ---- gate functions without a branch, for phases that evaluate many of them in one thread (the
 //      library's division and tanhf branch on rare operands, which keeps the units' chains from
-//      overlapping).  As accurate as those: a reciprocal refined by one Newton step, and tanh from
-//      its Taylor series below 1/2 (through x^15, the rest under 1e-8) and from exp above.
-//      NaN and infinities come out as the library's do, except that sigmoid falls no further
-//      than e^-80.
-__device__ __forceinline__ float recip_nb(float d) {  // 1 / d, 1 <= d <= 1e35 or NaN
+//      overlapping).  Over every fp32 argument their largest error against fp64 is no larger than the
+//      library's on any interval (tests/test_gpu_gate_functions.py): tanh at most 1.17 units of the last
+//      place (tanhf 1.82), sigmoid the same as 1 / (1 + expf(-x)) down to x = -87, below which it stays
+//      at e^-87.  A reciprocal refined by one Newton step; tanh below 1 from the polynomial of degree 8 in
+//      x^2 that interpolates (tanh(x) / x - 1) / x^2 at the Chebyshev nodes of [0, 1] (0.15 * 2^-24 of
+//      tanh left out), and from exp above, where what is subtracted from 1 is at most 0.24 (met at 1/2,
+//      as the Taylor series through x^15 allows, it is 0.54, and the error just past it 2.5 units).
+//      NaN and infinities come out as the library's do.
+__device__ __forceinline__ float recip_nb(float d) {  // 1 / d, 1 <= d < 2^126 or NaN
   const float r = __fdividef(1.f, d);
   return fmaf(r, fmaf(-d, r, 1.f), r);
 }
-__device__ __forceinline__ float sigmoid_nb(float x) { return recip_nb(1.f + expf(-x > 80.f ? 80.f : -x)); }
+__device__ __forceinline__ float sigmoid_nb(float x) { return recip_nb(1.f + expf(-x > 87.f ? 87.f : -x)); }
 __device__ __forceinline__ float tanh_nb(float x) {
   const float a = fabsf(x), s = x * x;
-  float t = -929569.f / 638512875.f;
-  t = fmaf(t, s, 21844.f / 6081075.f);
-  t = fmaf(t, s, -1382.f / 155925.f);
-  t = fmaf(t, s, 62.f / 2835.f);
-  t = fmaf(t, s, -17.f / 315.f);
-  t = fmaf(t, s, 2.f / 15.f);
-  t = fmaf(t, s, -1.f / 3.f);
+  float t = -4.846711090e-05f;
+  t = fmaf(t, s, 3.376898239e-04f);
+  t = fmaf(t, s, -1.242157537e-03f);
+  t = fmaf(t, s, 3.478386439e-03f);
+  t = fmaf(t, s, -8.826250210e-03f);
+  t = fmaf(t, s, 2.186257578e-02f);
+  t = fmaf(t, s, -5.396759510e-02f);
+  t = fmaf(t, s, 1.333333105e-01f);
+  t = fmaf(t, s, -3.333333433e-01f);
   const float small = fmaf(x * s, t, x);
   const float big = copysignf(fmaf(-2.f, recip_nb(1.f + expf(a > 40.f ? 80.f : 2.f * a)), 1.f), x);
-  return a < 0.5f ? small : big;
+  return a < 1.f ? small : big;
 }
 
 // Where unit c of a sequence's h_j lies in the CTA's shared memory: within each run of 256 units the
