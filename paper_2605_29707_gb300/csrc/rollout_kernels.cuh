@@ -1330,7 +1330,7 @@ __device__ __forceinline__ float lane_gumbel(unsigned long long seed, int lane, 
 // shared memory as 128-byte swizzled K-major tiles (loaded once by TMA); rows past those blocks
 // are read through L2 (RestTile; inverse CDF: on the CUDA cores).  u_j is the B operand: rows
 // 3b, 3b + 1 and 3b + 2 hold bf16 terms of u_j[b] that add up to it (u_terms), so that
-// D[:, 3b] + (D[:, 3b + 1] + D[:, 3b + 2]) is W2 u_j with u kept to fp32's 24 bits (three terms; two,
+// D[:, 3b] + (D[:, 3b + 1] + D[:, 3b + 2]) (join_terms) is W2 u_j with u kept to fp32's 24 bits (three terms; two,
 // 16 bits, under the inverse-CDF rule), accumulated in fp32.  Each block's MMAs go into its own kN columns of D (16, or 32 above
 // four sequences), issued by one thread of its own warp; the epilogue adds the staged base logit and
 // b2 of each row.
@@ -1361,6 +1361,13 @@ __device__ __forceinline__ void u_terms(float v, int terms, __nv_bfloat16 (&t)[3
   const float r1 = isfinite(hi) ? v - hi : 0.f;
   t[1] = __float2bfloat16_rn(r1);
   t[2] = __float2bfloat16_rn(terms > 2 ? r1 - __bfloat162float(t[1]) : 0.f);
+}
+
+// W2 u of a row from its products with u's terms.  An infinite weight makes the first one infinite, of the
+// sign that u gives it (or NaN); the other terms, of either sign, must not turn that into NaN.
+__device__ __forceinline__ float join_terms(float d0, float d1, float d2) {
+  const float rest = d1 + d2;
+  return d0 + (isfinite(d0) ? rest : 0.f);
 }
 
 // The first 3 KB accumulator columns (one row's dot products) from a D block's column address.
@@ -1444,12 +1451,12 @@ struct RestTile {
       if constexpr (KB <= 2) {
         const float x0 = __shfl_sync(0xffffffffu, acc[0][2 * h], (lane & ~3) | 2);
         const float x1 = __shfl_sync(0xffffffffu, acc[0][2 * h + 1], (lane & ~3) | 2);
-        d[h][0] = acc[0][2 * h] + (acc[0][2 * h + 1] + (t == 0 ? x0 : x1));
+        d[h][0] = join_terms(acc[0][2 * h], acc[0][2 * h + 1], t == 0 ? x0 : x1);
       } else if constexpr (KB == 4) {
-        d[h][0] = acc[0][2 * h] + (acc[0][2 * h + 1] + acc[1][2 * h]);
+        d[h][0] = join_terms(acc[0][2 * h], acc[0][2 * h + 1], acc[1][2 * h]);
       } else {
-        d[h][0] = acc[0][2 * h] + (acc[0][2 * h + 1] + acc[2][2 * h]);
-        d[h][1] = acc[1][2 * h] + (acc[1][2 * h + 1] + acc[2][2 * h + 1]);
+        d[h][0] = join_terms(acc[0][2 * h], acc[0][2 * h + 1], acc[2][2 * h]);
+        d[h][1] = join_terms(acc[1][2 * h], acc[1][2 * h + 1], acc[2][2 * h + 1]);
       }
     }
   }
@@ -1849,7 +1856,7 @@ __global__ void __launch_bounds__(kRollThreads, 1)
                   for (int b = 0; b < KB; ++b) {
                     if (b < B) {
                       const float logit =
-                          s_base[b * rows_cta + row] + s_b2[row] + (d[3 * b] + (d[3 * b + 1] + d[3 * b + 2]));
+                          s_base[b * rows_cta + row] + s_b2[row] + join_terms(d[3 * b], d[3 * b + 1], d[3 * b + 2]);
                       x[t][b] = logit;
                       if constexpr (kCdf) {
                         if (glg) glg[static_cast<size_t>(b) * V + r_lo + row] = logit;
