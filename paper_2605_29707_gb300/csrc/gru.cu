@@ -64,6 +64,10 @@ __device__ __forceinline__ uint4 ld_relaxed_v4(const uint32_t* p) {
   return v;
 }
 
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // Four state words all written in this step: their low halves equal the step's tag.
 __device__ __forceinline__ bool all_tagged(const uint4& v, uint32_t tag) {
   return (((v.x ^ tag) | (v.y ^ tag) | (v.z ^ tag) | (v.w ^ tag)) & 0xFFFFu) == 0u;
@@ -84,12 +88,13 @@ __device__ __forceinline__ bool poll_v4(const uint32_t* p, uint4& v, uint32_t ta
 }
 
 // Packed states (wide launches, whose state rows arrive cleared): eight bf16 values in 16 bytes, each
-// with bit 14 set once it is written.  A state is a convex combination of tanh values, so |h| <= 1
+// with bit 14 set once it is written; written and read in 32-bit words (two neighbouring units), as the
+// memory model orders accesses of one size only.  A state is a convex combination of tanh values, so |h| <= 1
 // and that exponent bit is free; NaN (0x7FC0) reads back as NaN because no |h| <= 1 has a code above
 // 0x3F80 below the bit.  Half the bytes of tagged words: what a step reads from L2 is what bounds it
 // at 16 and more sequences a CTA.
-__device__ __forceinline__ uint16_t packed_state(float h) {
-  return static_cast<uint16_t>(__bfloat16_as_ushort(__float2bfloat16_rn(h)) | 0x4000u);
+__device__ __forceinline__ uint32_t packed_state(float h) {
+  return __bfloat16_as_ushort(__float2bfloat16_rn(h)) | 0x4000u;
 }
 __device__ __forceinline__ bool all_written(const uint4& v) {
   return (v.x & v.y & v.z & v.w & 0x40004000u) == 0x40004000u;
@@ -862,8 +867,16 @@ __global__ void __launch_bounds__(kGruThreads, kX > 0 ? 1 : 2) gru_kernel(const 
         const float h = (1.f - z) * n + z * hp;
         hprev[bl * U + jl] = h;
         if (held && hold.x == kHoldPublish && hold.z == t) continue;  // test hook: withheld
-        if (kWide) __stcg(hxp + m * Ds + j, packed_state(h));
-        else p.hx[m * Ds + j] = tagged(h, tag);
+        if constexpr (kWide) {
+          // units 2 i and 2 i + 1 of a sequence lie in neighbouring lanes (Uc is a multiple of 8) and are
+          // published as one word, the size in which the other CTAs read them
+          const int live = nb * Uc - (warp * 32 + rr * kGruThreads);  // lanes of this warp with a pair
+          const uint32_t own = packed_state(h);
+          const uint32_t next = __shfl_down_sync(live >= 32 ? 0xffffffffu : (1u << live) - 1u, own, 1);
+          if ((lane & 1) == 0) st_relaxed(reinterpret_cast<uint32_t*>(hxp + m * Ds + j), own | (next << 16));
+        } else {
+          p.hx[m * Ds + j] = tagged(h, tag);
+        }
         if (p.s_out) p.s_out[m * Ds + j] = __float2bfloat16_rn(h);
       }
       __syncthreads();

@@ -1,0 +1,21 @@
+"""Properties of the CUDA sources that no run on one GPU can show (read from the text of csrc/, no GPU)."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_29707_gb300", "csrc")
+
+
+def _code(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_packed_states_are_published_in_the_size_they_are_read():
+    """The GRU's packed states cross CTAs without a barrier: the memory model orders a strong read with a
+    strong write of the same 32-bit word, and says nothing of a weak 16-bit write to half of it."""
+    code = _code("gru.cu")
+    assert "ld.relaxed.gpu.global.v4.u32" in code
+    assert re.search(r"hxp\s*\[|__st\w+\(\s*hxp", code) is None
+    stores = re.findall(r"(\w+)\(reinterpret_cast<(\w+)\*>\(hxp", code)
+    assert stores == [("st_relaxed", "uint32_t")], stores
+    assert re.search(r"st_relaxed\(uint32_t\*[^}]*st\.relaxed\.gpu\.global\.u32", code)
