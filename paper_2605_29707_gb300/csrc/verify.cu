@@ -433,13 +433,8 @@ cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, con
   const int slice = ((V + kSplit - 1) / kSplit + 3) & ~3;
   if (slice > kMaxSampleSlice) return cudaErrorInvalidValue;
   const size_t smem = static_cast<size_t>(slice) * sizeof(float);
-  static bool attr_set = false;  // the largest staging size is set once per process
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(row_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               kMaxSampleSlice * static_cast<int>(sizeof(float)));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(row_sample_kernel), smem, true);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(rows * kSplit));
   cfg.blockDim = dim3(kSampleThreads);
@@ -452,8 +447,8 @@ cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, con
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, row_sample_kernel, logits, V, inv_t, uniforms, row_sample, kAhead,
-                                     g_held_row.exchange(-1));
+  e = cudaLaunchKernelEx(&cfg, row_sample_kernel, logits, V, inv_t, uniforms, row_sample, kAhead,
+                         g_held_row.exchange(-1));
   if (e != cudaSuccess) return e;
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -19,3 +19,12 @@ def test_packed_states_are_published_in_the_size_they_are_read():
     stores = re.findall(r"(\w+)\(reinterpret_cast<(\w+)\*>\(hxp", code)
     assert stores == [("st_relaxed", "uint32_t")], stores
     assert re.search(r"st_relaxed\(uint32_t\*[^}]*st\.relaxed\.gpu\.global\.u32", code)
+
+
+def test_kernel_attributes_are_set_per_device():
+    """A kernel's attributes belong to a device: only ensure_smem_attr, which keeps what it set by (device,
+    kernel) under a lock, sets them, and no launch keeps a flag for the whole process."""
+    for name in sorted(os.listdir(CSRC)):
+        code = _code(name)
+        assert code.count("cudaFuncSetAttribute(") == (2 if name == "api.cu" else 0), name
+        assert re.search(r"static\s+bool\s+\w+\s*=", code) is None, name
