@@ -27,8 +27,13 @@
 namespace dm {
 
 constexpr int kArgmaxThreads = 256;
-constexpr int kSplit = 8;        // CTAs (one cluster) per row
-constexpr int kSplitRows = 152;  // from this many rows on (one an SM) the argmax takes two CTAs a row
+constexpr int kSplit = 8;  // CTAs (one cluster) per row
+
+static cudaError_t sm_count(int* sms) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
 
 __device__ __forceinline__ uint32_t dsmem_addr(const void* local, uint32_t rank) {
   uint32_t r;
@@ -193,7 +198,7 @@ static cudaError_t launch_walk(const int32_t* parent, const int32_t* token, cons
 // ------------------------------------------------------------------------------ row draw
 constexpr int kSampleThreads = 256;
 constexpr int kStageChunks = 4;  // bulk copies that stage a CTA's slice
-constexpr int kAhead = 56;       // rows: what is resident at once (three CTAs an SM, eight a row)
+constexpr int kAheadCtas = 3;    // a CTA asks for the slice that many CTAs an SM further on (see the launch)
 
 __device__ __forceinline__ float ld_cluster_f32(const void* local, uint32_t rank) {
   float v;
@@ -435,6 +440,14 @@ cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, con
   const size_t smem = static_cast<size_t>(slice) * sizeof(float);
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(row_sample_kernel), smem, true);
   if (e != cudaSuccess) return e;
+  // How many rows ahead a CTA's slice is brought into L2: three CTAs an SM, what is resident at once at
+  // V = 151936.  It is no less at smaller vocabularies, where more are resident: at V = 32000 and 64000
+  // the rows resident there (151, 75) took 35.4 us for 544 rows and 148 for 2112, three CTAs an SM 34.5
+  // and 146.
+  int sms = 0;
+  e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const int ahead = kAheadCtas * sms / kSplit;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(rows * kSplit));
   cfg.blockDim = dim3(kSampleThreads);
@@ -447,7 +460,7 @@ cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, con
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, row_sample_kernel, logits, V, inv_t, uniforms, row_sample, kAhead,
+  e = cudaLaunchKernelEx(&cfg, row_sample_kernel, logits, V, inv_t, uniforms, row_sample, ahead,
                          g_held_row.exchange(-1));
   if (e != cudaSuccess) return e;
   e = cudaGetLastError();
@@ -484,8 +497,11 @@ cudaError_t launch_verify_greedy(const float* logits, const int32_t* parent, con
   // longer runs and launch a quarter of the clusters (V = 151936: 17 rows 11.0 us against 12.4 split in
   // two, 68 rows 11.0 against 14.4; 272 rows 38.3 against 32.9, 2112 rows 208 against 185.5 us, the
   // measured copy rate).
-  const cudaError_t e = rows < kSplitRows ? launch_row_argmax<kSplit>(logits, V, row_argmax, rows, stream)
-                                          : launch_row_argmax<2>(logits, V, row_argmax, rows, stream);
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  e = rows < sms ? launch_row_argmax<kSplit>(logits, V, row_argmax, rows, stream)
+                 : launch_row_argmax<2>(logits, V, row_argmax, rows, stream);
   if (e != cudaSuccess) return e;
   return launch_walk(parent, token, row_argmax, B, N, nodes, count, bonus, stream);
 }

@@ -28,3 +28,11 @@ def test_kernel_attributes_are_set_per_device():
         code = _code(name)
         assert code.count("cudaFuncSetAttribute(") == (2 if name == "api.cu" else 0), name
         assert re.search(r"static\s+bool\s+\w+\s*=", code) is None, name
+
+
+def test_sizes_of_the_chip_come_from_the_device():
+    """No launch rule names the SM count of one chip: it is read from the device (api.cu's 152 is what
+    domino_launches_per_step answers for where none is visible)."""
+    for name in sorted(os.listdir(CSRC)):
+        found = re.findall(r"\b152\b", _code(name))
+        assert len(found) == (1 if name == "api.cu" else 0), (name, found)
