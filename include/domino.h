@@ -179,7 +179,7 @@ DOMINO_API int domino_check_status(const void* workspace, void* stream);
  *   DOMINO_HOLD_STATE          CTA gru_cta does not publish its hidden states of position
  *                              `step` (0 <= step < 64; a step >= K withholds nothing);
  *   DOMINO_HOLD_CLEAR_BARRIER  CTA gru_cta does not arrive at the barrier of the state clear
- *                              that a small-batch step (B <= 2 at K = 16) runs when the workspace
+ *                              that a small-batch step (one of three launches) runs when the workspace
  *                              last held another kind or shape of step (or is fresh); `step` is
  *                              ignored, and a step that needs no clear withholds nothing;
  *   DOMINO_HOLD_ROW_COPY       the next domino_verify_tree_sample launch does not copy part of row
@@ -209,8 +209,9 @@ DOMINO_API int domino_abi_version(void);
 /* Number of kernel launches one domino_draft_step makes for these sizes (head on when
  * R > 0), so a caller can count device work: the plan of the current device (of a 152-SM GB300
  * when no device is visible).  3 with the head off, 3 for small batches whose GRU computes its
- * own projections (B <= 2 at K = 16), 6 for other batches of at most 128 positions, 7 above;
- * a negative code for sizes domino_draft_step would reject. */
+ * own projections (with d_s = 1024: up to 32 positions at r = 256, 64 at 128, 128 below), 6 for
+ * other batches of at most 128 positions, 7 above; a negative code for sizes domino_draft_step
+ * would reject. */
 DOMINO_API int domino_launches_per_step(int B, int K, int H, int V, int Ds, int R, int k, int N);
 /* The same count for a head that carries an input-projection table (head->x_table): one launch
  * fewer wherever domino_launches_per_step counts an X GEMM (5 instead of 6, 6 instead of 7). */

@@ -1,7 +1,8 @@
 // api.cu -- host side of the C ABI declared in include/domino.h: argument checks, the launch
 // plan for the current device, workspace layout, TMA tensor maps and the launch sequence.
 //
-// Launch sequence of one step (all on the caller's stream).  Small batches (B <= 2 at K = 16):
+// Launch sequence of one step (all on the caller's stream).  Small batches (at r = 256 and d_s = 1024,
+// up to 32 positions; up to 128 at a smaller r, see `fused` in the plan):
 //   gru      prologue: prefix-id check, E . W_ih^T from the embedding rows by id (or rows of the
 //            input-projection table) and hidden . W1[:, :H]^T; then S_j = GRU(E_0..E_j) and
 //            u = SiLU(. + S . W1[:, H:]^T + b1)  (cooperative; its first CTA resets the status)
@@ -214,8 +215,8 @@ int make_plan_sms(int B, int K, int H, int V, int Ds, int R, int k, int N, bool 
     p.gru = dm::gru_plan(B, Ds, sms);
     if (p.gru.smem == 0) return DOMINO_ERR_UNSUPPORTED;
     // Overlap the GRU with the W_lm stream when a deferred-mode vocab CTA and a GRU CTA fit on
-    // one SM (228 KB of shared memory, 1 KB reserved per CTA) and every tile of a CTA can keep
-    // its own TMEM accumulator until u is ready.
+    // one SM (228 KB of shared memory, 1 KB reserved per CTA); the first tiles of a CTA then keep
+    // their accumulators in tensor memory until u is ready (defer_tiles, below).
     const int vsm = dm::tc_softmax_deferred_smem(p.bn, p.kmax);
     p.overlap = p.u_in_gru && vsm > 0 && static_cast<size_t>(vsm) + p.gru.smem + 2048 <= 228 * 1024;
     // Equal chunks on the wide accumulator blocks, whose tiles' epilogues count (us, whole against

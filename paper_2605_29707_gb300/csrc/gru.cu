@@ -464,7 +464,7 @@ __device__ __forceinline__ bool u_dots(const GruParams& p, const __nv_bfloat16* 
 }
 
 // At most 128 registers per thread (two CTAs' worth per SM), so that a GRU CTA and a vocabulary
-// GEMM CTA (at most 168 registers x 192 threads) fit in one SM's register file.
+// GEMM CTA (at most 128 registers, six warps counted as eight) fit in one SM's register file.
 // kTable: the input-gate sums come from the input-projection table (p.x_table) rather than
 // from xs (a separate instantiation, so that the path without a table keeps its registers).
 // kX > 0 (wide): a launch that shares no SM with the vocabulary GEMM (large batches): the register

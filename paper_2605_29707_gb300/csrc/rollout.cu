@@ -8,7 +8,7 @@ namespace dm {
 
 // ================================================================ launch
 // Resident kernel: shared-memory W2 rows that fit beside u, the staged base logits and `extra`
-// bytes (h_j of every sequence for two-barrier steps); -1 when those alone do not fit.
+// bytes (h_j of every sequence for one-barrier steps); -1 when those alone do not fit.
 static int resident_smem_rows(int B, int V, int R, int grid, long long extra = 0) {
   const int rows_cta = resident_rows_per_cta(V, grid);
   const long long fixed =
@@ -32,12 +32,12 @@ size_t rollout_smem_bytes(int B, int V, int R, bool head, int grid) {
          static_cast<size_t>(B) * rollout_rows_per_cta(V, R, head, grid) * sizeof(float);
 }
 
-// Shared memory of h_j of every sequence (two-barrier steps): whole 256-unit runs (h_slot), and 16
+// Shared memory of h_j of every sequence (one-barrier steps): whole 256-unit runs (h_slot), and 16
 // bytes for its alignment.
 static long long h_bytes(const RolloutParams& p) { return static_cast<long long>(p.B) * ((p.Ds + 255) / 256 * 256) * 4 + 16; }
 
-// Two grid barriers per step (phase A done by every CTA for all units, gates_all / ub_phase):
-// the resident kernel with a table, when h_j of every sequence fits in shared memory beside u and
+// One grid barrier per step, and a wait for u's rows (phase A done by every CTA for all units,
+// gates_all / ub_phase): the resident kernel with a table, when h_j of every sequence fits in shared memory beside u and
 // the base logits (the shared-memory W2 rows give way to it).
 static bool use_fast_gates(const RolloutParams& p, int grid) {
   // gates_all reads the biases four at a time (8-byte loads)

@@ -572,8 +572,8 @@ __device__ __forceinline__ float tanh_nb(float x) {
 // warp's two 16-byte reads of its groups (ub_rows) touch every bank once each.
 __device__ __forceinline__ int h_slot(int c) { return (c & ~255) | ((c & 4) << 5) | ((c & 0xF8) >> 1) | (c & 3); }
 
-// ---- phase A with the input-projection table, two barriers per step (resident kernel): every
-//      CTA computes h_j of every unit and sequence itself, so that no grid barrier follows.  The
+// ---- phase A of the one-barrier step (resident kernel with the input-projection table): every CTA
+//      computes h_j of every unit and sequence itself, so that no grid barrier follows.  The
 //      input-gate sums are row t_j of the table, the recurrent sums W_hh h_{j-1} were computed in
 //      the previous step's phase B (gh; none at j = 0), and h_{j-1} is the CTA's own copy in
 //      shared memory, updated in place (unit q of h_j needs unit q of h_{j-1} only); four consecutive
@@ -775,7 +775,7 @@ __device__ __forceinline__ void ub_phase(const RolloutParams& p, int j, const fl
 //      = b K + j and rank row q, the half of u's argument that does not depend on the
 //      recurrence.  Warp w takes row q = w % R and the positions m = w / R, w / R + G, ...
 //      (G = max(1, warps / R)), four at a time, so a W1 row is read once per four positions.
-//      The caller then counts its CTA in p.uhcount (release): the two-barrier step reads uh
+//      The caller then counts its CTA in p.uhcount (release): the one-barrier step reads uh
 //      before any grid barrier, so its first phase B acquires that count instead.
 static __device__ void uh_prologue(const RolloutParams& p, int gw, int nwarps, int lane, uint64_t pol) {
   const int H = p.H, Ds = p.Ds, R = p.R, M = p.B * p.K;
@@ -1464,7 +1464,7 @@ struct RestTile {
 
 // kCdf (kMma only): the inverse-CDF rule, whose rows past the MMA blocks stay on the CUDA cores and
 // whose sums keep their order, since they decide the draws.
-// kFast: the two-barrier step (p.fast_gates); otherwise the three-phase one.  Separate kernels, since
+// kFast: the one-barrier step (p.fast_gates); otherwise the three-phase one.  Separate kernels, since
 // each needs the whole register budget.
 template <int KB, bool kMma, bool kRace, bool kCdf, bool kFast>
 __global__ void __launch_bounds__(kRollThreads, 1)
@@ -1501,7 +1501,7 @@ __global__ void __launch_bounds__(kRollThreads, 1)
                     : reinterpret_cast<float*>(s_dyn + static_cast<size_t>(p.smem_rows) * R * 2);  // [B][R]
   float* s_base = s_u + B * R;                                                          // [B][rows_cta]
   float* s_b2 = s_base + B * rows_cta;                                                  // [rows_cta]
-  // [B][Ds] h_j of every sequence (two-barrier steps only), 16-byte aligned for vector reads
+  // [B][Ds] h_j of every sequence (one-barrier steps only), 16-byte aligned for vector reads
   float* s_h = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(s_b2 + rows_cta) + 15) & ~static_cast<uintptr_t>(15));
   __shared__ __align__(8) uint64_t s_fill;  // the shared-memory rows landed
   __shared__ __align__(8) uint64_t s_mma;   // kMma: this step's MMAs completed
@@ -1635,7 +1635,7 @@ __global__ void __launch_bounds__(kRollThreads, 1)
       const float* hprev = p.h + static_cast<size_t>((j + 1) & 1) * B * p.Ds;  // h_{j-1} (zeros at j = 0)
       float* hcur = p.h + static_cast<size_t>(j & 1) * B * p.Ds;
       // this step's base logits for the CTA's rows: asynchronous copies that land during A and B
-      // (greedy two-barrier step: issued by the previous step's finish, from step 1 on)
+      // (greedy one-barrier step: issued by the previous step's finish, from step 1 on)
       if (j == 0 || p.best == nullptr || !kFast) {
         copy_base(p, j, s_base, r_lo, r_n, rows_cta);
       }
@@ -2181,7 +2181,7 @@ static cudaError_t launch_coop(Kern kern, const RolloutParams& p, int grid, int 
 }
 
 // The resident kernel's instantiations, each set in a unit of its own (rollout_resident_*.cu) so that
-// they compile in parallel: two-barrier and three-phase steps of the greedy (and, on the CUDA cores,
+// they compile in parallel: one-barrier and three-phase steps of the greedy (and, on the CUDA cores,
 // inverse-CDF) loop and of the race, and the inverse-CDF loop's tensor-core layout.
 #define DM_ROLL_LAUNCH(name) \
   cudaError_t name(const RolloutParams& p, int grid, size_t smem, cudaStream_t stream, const CUtensorMap& tm)

@@ -1,4 +1,4 @@
-// rollout_resident_fast.cu -- the resident kernel's two-barrier steps: greedy and inverse-CDF loops.
+// rollout_resident_fast.cu -- the resident kernel's one-barrier steps: greedy and inverse-CDF loops.
 #include "rollout_kernels.cuh"
 
 namespace dm {

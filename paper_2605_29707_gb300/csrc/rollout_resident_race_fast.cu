@@ -1,4 +1,4 @@
-// rollout_resident_race_fast.cu -- the resident kernel's two-barrier steps: the exponential race.
+// rollout_resident_race_fast.cu -- the resident kernel's one-barrier steps: the exponential race.
 #include "rollout_kernels.cuh"
 
 namespace dm {

@@ -177,8 +177,8 @@ __global__ void __launch_bounds__(32) tree_walk_kernel(const int32_t* __restrict
   }
 }
 
-// The walk, launched as a programmatic dependent of the row kernel before it: its launch and the
-// clearing of the accepted-node list overlap the row kernel's tail.
+// The walk, launched as a programmatic dependent of the row kernel before it, which triggers it by
+// exiting: the launch, not the walk's work, overlaps the row kernel's last CTAs.
 static cudaError_t launch_walk(const int32_t* parent, const int32_t* token, const int32_t* row_choice, int B,
                                int N, int32_t* nodes, int32_t* count, int32_t* bonus, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
