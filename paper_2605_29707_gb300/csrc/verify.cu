@@ -438,7 +438,7 @@ cudaError_t launch_verify_sample(const float* logits, const int32_t* parent, con
   const int slice = ((V + kSplit - 1) / kSplit + 3) & ~3;
   if (slice > kMaxSampleSlice) return cudaErrorInvalidValue;
   const size_t smem = static_cast<size_t>(slice) * sizeof(float);
-  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(row_sample_kernel), smem, true);
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(row_sample_kernel), smem, false);
   if (e != cudaSuccess) return e;
   // How many rows ahead a CTA's slice is brought into L2: three CTAs an SM, what is resident at once at
   // V = 151936.  It is no less at smaller vocabularies, where more are resident: at V = 32000 and 64000
